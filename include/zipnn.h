@@ -81,24 +81,22 @@ typedef struct zipnn_stream {
 /* Decoder launch parameters for batched decoding.  Zero fields take defaults;
  * the values change speed only, never the decoded bytes. */
 typedef struct zipnn_tuning {
-    int32_t threads;      /* decoder threads per CTA: 128 or 256 (0 = 256);
-                             256 applies to batches of one dtype with W >= 11
-                             whose lane counts are all multiples of 256;
-                             otherwise, and for any other value, 128 */
+    int32_t threads;      /* decoder threads per CTA: 128 or 256 (0 = 256); 256
+                             applies when some tensor has more than 128
+                             sub-streams per work item; otherwise, and for any
+                             other value, 128 */
     int32_t ctas_per_sm;  /* resident CTAs per SM for the persistent grid */
-    int32_t lut_bits;     /* decode table width W in bits: 10, 11 or 12 (0 = 12);
-                             W = 10 resolves codes longer than 10 bits through
-                             the canonical limits, W = 11 resolves 12-bit codes
-                             inside the table */
+    int32_t lut_bits;     /* accepted and ignored: the decode tables are indexed
+                             by 12 bits, the longest code (narrower tables were
+                             never faster) */
     int32_t debug_flags;  /* 0.  Bit 0 is fault injection for tests: the decoder
                              waits for 16 bytes that are never copied, so its
                              bounded wait gives up after 100 ms and the call
                              reports ZIPNN_ETIMEOUT via zipnn_sync_status */
     int32_t parts;        /* work items per chunk: 0 = automatic (launches whose
                              chunks would fill at most half the SMs split each
-                             model-weight chunk's sub-streams over 2, 4 or 8
-                             work items of 128-thread CTAs), 1 = never split,
-                             2, 4 or 8 = split whenever the lanes allow */
+                             chunk's sub-streams over 2, 4 or 8 work items),
+                             1 = never split, 2, 4 or 8 = always */
 } zipnn_tuning;
 
 /* Library version (the container version is 1). */
@@ -250,8 +248,9 @@ zipnn_status zipnn_decompressed_size(const zipnn_stream* s, size_t* nbytes, int*
 zipnn_status zipnn_decompress(const zipnn_stream* s, const void* d_base_or_null, void* d_dst,
                               size_t dst_nbytes, void* cuda_stream);
 
-/* Decompress count containers in ONE persistent kernel that pulls
- * (tensor, chunk) work items from a device queue (the batching form).  Each
+/* Decompress count containers in one persistent kernel per dtype family (BF16
+ * and FP16 share one) that pulls (tensor, chunk) work items from a device queue
+ * (the batching form).  Each
  * container decodes to exactly its original bytes (Sec. 2.3), as with
  * zipnn_decompress; the chunk maps (Sec. 5.1, "Metadata and parallelism") make
  * every chunk of every container an independent work item, which is what
@@ -275,7 +274,7 @@ zipnn_status zipnn_batch_decompress(const zipnn_stream* streams, const void* con
  * zipnn_plan_decompress: the persistent decoder over all containers (work
  *   items pulled from a device ticket), as zipnn_batch_decompress.  Creation
  *   reads the containers' chunk maps (a device-to-host copy) to size the
- *   decoder's shared-memory stage and pick its kernel variant; maps that
+ *   decoder's shared-memory stage; maps that
  *   change later change the speed, never the decoded bytes.
  * zipnn_plan_compress: the four encoder kernels over all tensors, as
  *   zipnn_batch_compress_into, with the scratch owned by the plan.

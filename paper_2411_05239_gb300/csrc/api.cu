@@ -463,10 +463,9 @@ zipnn_status zipnn_decompress(const zipnn_stream* s, const void* d_base_or_null,
   if (!err) return ZIPNN_ECUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   Job J = decode_job(s, d_base_or_null, d_dst);
-  cudaError_t e = launch_decode_ex(nullptr, &J, 1, J.n_chunks, (int)s->n_groups, nullptr, err,
-                                   nullptr, st, s->dtype, s->chunk_bytes, s->lanes % 256 == 0,
-                                   stage_frac64(s->dtype, s->flags),
-                                   (s->flags & ZIPNN_FLAG_DELTA) != 0, false, 0u, s->lanes);
+  DecodeShape shape;
+  shape.add(s->dtype, s->flags, s->chunk_bytes, s->lanes);
+  cudaError_t e = launch_decode_ex(nullptr, &J, 1, J.n_chunks, shape, nullptr, err, nullptr, st);
   return cuda_status(e);
 }
 
@@ -476,20 +475,9 @@ zipnn_status zipnn_batch_decompress(const zipnn_stream* streams, const void* con
   if (count < 0 || (count > 0 && (!streams || !d_dsts))) return ZIPNN_EINVAL;
   if (count == 0) return ZIPNN_OK;
   std::vector<Job> jobs((size_t)count);
-  uint64_t chunk = 0, max_chunk = 0;
-  int max_groups = 1;
-  int uniform = streams[0].dtype;
-  bool lanes256 = true, has_delta = false;
-  int frac64 = 0;
-  uint32_t common_lanes = streams[0].lanes;
+  std::vector<uint64_t> chunks((size_t)count);
   for (int i = 0; i < count; i++) {
     const zipnn_stream* s = &streams[i];
-    if (s->lanes != common_lanes) common_lanes = 0;
-    if (s->flags & ZIPNN_FLAG_DELTA) has_delta = true;
-    if (s->dtype != uniform) uniform = -1;
-    if (s->chunk_bytes > max_chunk) max_chunk = s->chunk_bytes;
-    if (s->lanes % 256) lanes256 = false;
-    if (stage_frac64(s->dtype, s->flags) > frac64) frac64 = stage_frac64(s->dtype, s->flags);
     zipnn_status rc = check_stream(s);
     if (rc) return rc;
     const void* base = d_bases ? d_bases[i] : nullptr;
@@ -497,27 +485,26 @@ zipnn_status zipnn_batch_decompress(const zipnn_stream* streams, const void* con
     if ((s->orig_nbytes && !d_dsts[i]) || !aligned16(d_dsts[i]) || !aligned16(base))
       return ZIPNN_EINVAL;
     jobs[i] = decode_job(s, base, d_dsts[i]);
-    jobs[i].chunk_begin = chunk;
-    chunk += jobs[i].n_chunks;
-    if ((int)s->n_groups > max_groups) max_groups = (int)s->n_groups;
+    chunks[i] = jobs[i].n_chunks;
   }
+  DecodeGroup groups[kDecodeFamilies];
+  const int ngroups = group_decode_jobs(jobs, chunks, groups);
   uint32_t* err = err_word();
   if (!err) return ZIPNN_ECUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   void* dmem = nullptr;
   const size_t tbytes = sizeof(Job) * (size_t)count;
-  cudaError_t e = cudaMallocAsync(&dmem, tbytes + 16, st);
+  constexpr size_t kTicketBytes = 2 * sizeof(unsigned long long) * kDecodeFamilies;
+  cudaError_t e = cudaMallocAsync(&dmem, tbytes + kTicketBytes, st);
   if (e != cudaSuccess) return cuda_status(e);
   Job* d_jobs = static_cast<Job*>(dmem);
   unsigned long long* d_ticket = reinterpret_cast<unsigned long long*>(static_cast<uint8_t*>(dmem) + tbytes);
-  // the job table and the two zeroed work-queue counters after it, in one copy
-  std::vector<uint8_t> up(tbytes + 16, 0);
+  // the job table and the zeroed work-queue counters after it, in one copy
+  std::vector<uint8_t> up(tbytes + kTicketBytes, 0);
   memcpy(up.data(), jobs.data(), tbytes);
   e = g_ring.h2d(d_jobs, up.data(), up.size(), st);
   if (e == cudaSuccess)
-    e = launch_decode_ex(d_jobs, nullptr, count, chunk, max_groups, tuning, err, d_ticket, st,
-                         uniform, max_chunk, lanes256, frac64, has_delta, false, 0u,
-                         common_lanes);
+    e = launch_decode_groups(d_jobs, groups, ngroups, tuning, err, d_ticket, st);
   cudaFreeAsync(dmem, st);
   return cuda_status(e);
 }

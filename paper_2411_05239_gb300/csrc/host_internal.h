@@ -4,6 +4,8 @@
 #pragma once
 #include <cstddef>
 #include <cstdint>
+#include <vector>
+
 #include <cuda_runtime.h>
 
 #include "zipnn.h"
@@ -55,21 +57,50 @@ cudaError_t launch_encode(const Job* d_jobs, const Job* h_one, int njobs, uint64
                           bool any_delta = false);
 bool fused_encoder_applies(int dtype, bool any_skip);
 
-// Decoder (decode.cu): one persistent launch over all chunks of the jobs.
+// Decoder (decode.cu): one persistent launch per dtype family over all chunks
+// of its jobs.  What a launch needs to know of its jobs, gathered with add():
+struct DecodeShape {
+  int family = ZIPNN_BF16; // dtype_family of every job
+  int max_groups = 1;
+  uint64_t max_chunk = 0;
+  uint32_t max_lanes = 1, min_lanes = ZIPNN_MAX_LANES;
+  bool delta = false;      // some job has a base
+  int frac64 = 0;          // payload bytes as a fraction of the largest chunk (stage_frac64)
+  uint32_t stage_need = 0; // stage bytes measured from the chunk maps (0 = use frac64)
+  void add(int dtype, uint32_t flags, uint32_t chunk_bytes, uint32_t lanes) {
+    const int g = elem_size(dtype), q = stage_frac64(dtype, flags);
+    family = dtype_family(dtype);
+    if (g > max_groups) max_groups = g;
+    if (chunk_bytes > max_chunk) max_chunk = chunk_bytes;
+    if (lanes > max_lanes) max_lanes = lanes;
+    if (lanes < min_lanes) min_lanes = lanes;
+    if (flags & ZIPNN_FLAG_DELTA) delta = true;
+    if (q > frac64) frac64 = q;
+  }
+};
 // d_ticket: the device work queue, two 64-bit counters that must be zero
 // before the first launch on them (the kernel's last CTA zeroes them again),
-// or nullptr for a static assignment of chunks to CTAs.  frac64: stage size as a fraction of
-// the largest chunk (stage_frac64); has_delta: some job has a base; general:
-// use the general fast loops (two coded groups, SPARSE first groups) even
-// without a delta; stage_need: a stage size measured from the chunk maps (0 =
-// use frac64); common_lanes: the lanes of every job, or 0 if they differ (a
-// launch with few chunks may then split each chunk over several work items).
+// or nullptr for a static assignment of work items to CTAs.
 cudaError_t launch_decode_ex(const Job* d_jobs, const Job* h_one, int njobs,
-                             uint64_t nchunks_total, int max_groups, const zipnn_tuning* tuning,
-                             uint32_t* d_err, unsigned long long* d_ticket, cudaStream_t st,
-                             int uniform_dtype, uint64_t max_chunk, bool lanes256, int frac64,
-                             bool has_delta, bool general, uint32_t stage_need,
-                             uint32_t common_lanes);
+                             uint64_t nchunks_total, const DecodeShape& shape,
+                             const zipnn_tuning* tuning, uint32_t* d_err,
+                             unsigned long long* d_ticket, cudaStream_t st);
+// Batches: the jobs of one launch.
+constexpr int kDecodeFamilies = 3;
+struct DecodeGroup {
+  int first = 0, count = 0;
+  uint64_t nchunks = 0;
+  DecodeShape shape;
+};
+// Reorders the jobs by dtype family (keeping their order within one), numbers
+// their chunks (job i decodes chunks[i] of them) and fills groups[0..n), at
+// most kDecodeFamilies; returns n.  A family of empty tensors has no group.
+int group_decode_jobs(std::vector<Job>& jobs, const std::vector<uint64_t>& chunks,
+                      DecodeGroup* groups);
+// Launches every group; d_tickets: two counters each (see launch_decode_ex).
+cudaError_t launch_decode_groups(const Job* d_jobs, const DecodeGroup* groups, int ngroups,
+                                 const zipnn_tuning* tuning, uint32_t* d_err,
+                                 unsigned long long* d_tickets, cudaStream_t st);
 
 // Sub-streams per group-chunk when a call gives none: chunk_bytes / 512 for
 // plain 16-bit containers (two sub-streams per thread of a 256-thread decoder

@@ -4,6 +4,7 @@
 // cudaGraphLaunch.  This is the batching form of the codec: many tensors of
 // uneven sizes in one launch per kernel (ZipNN Sec. 5.1: chunks and byte groups
 // are independent, so one grid serves them all).
+#include <algorithm>
 #include <cstdint>
 #include <cstring>
 #include <vector>
@@ -33,21 +34,17 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 // What a decode launch needs, read from its containers' chunk maps: per chunk
 // the shared-memory stage that holds its coded (HUFF / SPARSE) payloads, 16-B
 // padded, plus 32 B and the table of every coded group after the first (the
-// decoder's staging rule), and whether a chunk takes the general fast loops
-// (two coded groups, or a SPARSE first group).
+// decoder's staging rule).
 struct MapNeed {
   uint64_t max_stage = 0;  // largest per-chunk need
   uint64_t chunks = 0;     // chunks seen
   uint64_t over = 0;       // chunks whose need exceeds the default stage
-  bool general = false;
 };
 
-void add_map_need(const uint8_t* map, uint32_t n_chunks, uint32_t G, int w, uint64_t dflt,
-                  MapNeed* nd) {
+void add_map_need(const uint8_t* map, uint32_t n_chunks, uint32_t G, uint64_t dflt, MapNeed* nd) {
   for (uint32_t c = 0; c < n_chunks; c++) {
     uint64_t used = 0;
     uint32_t ncoded = 0;
-    bool sparse0 = false;
     for (uint32_t g = 0; g < G; g++) {
       const uint8_t* e = map + ((uint64_t)c * G + g) * kEntryBytes;
       uint32_t size;
@@ -56,30 +53,23 @@ void add_map_need(const uint8_t* map, uint32_t n_chunks, uint32_t G, int w, uint
       if (mode == kHuff || mode == kSparse) {
         used += align_up(size, 16);
         ncoded++;
-        if (g == 0 && mode == kSparse) sparse0 = true;
       }
     }
     nd->chunks++;
     if (ncoded) {
-      const uint64_t need = used + 32 + (uint64_t)(ncoded - 1) * (4u << w);
+      const uint64_t need = used + 32 + (uint64_t)(ncoded - 1) * 4u * kLutSize;
       if (need > nd->max_stage) nd->max_stage = need;
       if (need > dflt) nd->over++;
     }
-    if (ncoded >= 2 || sparse0) nd->general = true;
   }
 }
 
 // The stage a plan asks for: 0 (the launcher's default rule) while the default
 // stage holds the payloads of at least 99% of the chunks, else the largest
-// need (which may leave one CTA per SM: the only way to stage such chunks).
+// need (which the launcher takes as far as two CTAs still share an SM).
 uint32_t planned_stage(const MapNeed& nd) {
   if (nd.over * 100 <= nd.chunks) return 0;
   return (uint32_t)(nd.max_stage > 0xFFFFFFFFull ? 0xFFFFFFFFull : nd.max_stage);
-}
-
-int plan_lut_bits(const zipnn_tuning* tuning) {
-  int w = (tuning && tuning->lut_bits) ? tuning->lut_bits : 12;
-  return w < 10 ? 10 : (w > 12 ? 12 : w);
 }
 
 zipnn_status fail(zipnn_plan* p, cudaError_t e) {
@@ -125,12 +115,8 @@ static zipnn_status plan_decode_range(const zipnn_stream* streams, const void* c
   if (!out || count <= 0 || !streams || !d_dsts || lo > hi) return ZIPNN_EINVAL;
   *out = nullptr;
   std::vector<Job> jobs;
-  std::vector<const zipnn_stream*> used;
-  uint64_t chunk = 0, max_chunk = 0, g = 0;
-  int max_groups = 1;
-  int uniform = -2;
-  bool lanes256 = true, has_delta = false;
-  int frac64 = 0;
+  std::vector<uint64_t> chunks;
+  uint64_t chunk = 0, g = 0;
   for (int i = 0; i < count; i++) {
     const zipnn_stream* s = &streams[i];
     if (s->n_groups != (uint32_t)elem_size(s->dtype) || s->dtype < 0 || s->dtype > ZIPNN_U8 ||
@@ -145,11 +131,6 @@ static zipnn_status plan_decode_range(const zipnn_stream* streams, const void* c
     const void* base = d_bases ? d_bases[i] : nullptr;
     if (((s->flags & ZIPNN_FLAG_DELTA) != 0) != (base != nullptr)) return ZIPNN_EINVAL;
     if (!d_dsts[i] || !aligned16(d_dsts[i]) || !aligned16(base)) return ZIPNN_EINVAL;
-    if (s->flags & ZIPNN_FLAG_DELTA) has_delta = true;
-    uniform = (uniform == -2 || uniform == s->dtype) ? s->dtype : -1;
-    if (s->chunk_bytes > max_chunk) max_chunk = s->chunk_bytes;
-    if (s->lanes % 256) lanes256 = false;
-    if (stage_frac64(s->dtype, s->flags) > frac64) frac64 = stage_frac64(s->dtype, s->flags);
     const uintptr_t shift = (uintptr_t)(a * s->chunk_bytes);
     Job J;
     memset(&J, 0, sizeof(J));
@@ -164,36 +145,36 @@ static zipnn_status plan_decode_range(const zipnn_stream* streams, const void* c
     J.dtype = s->dtype;
     J.flags = s->flags;
     J.stream_bytes = s->nbytes;
-    J.chunk_begin = chunk;
     J.chunk0 = (uint32_t)a;
     chunk += b - a;
-    if ((int)s->n_groups > max_groups) max_groups = (int)s->n_groups;
     jobs.push_back(J);
-    used.push_back(s);
+    chunks.push_back(b - a);
   }
   if (hi > g) return ZIPNN_EINVAL;
   if (jobs.empty()) return ZIPNN_EINVAL;  // nothing to decode in the range
   const int njobs = (int)jobs.size();
-  // stage and kernel variant from the chunk maps present now
-  MapNeed nd;
-  {
-    const int w = plan_lut_bits(tuning);
-    const uint64_t dflt = max_chunk * (uint64_t)frac64 / 64 + 1024;
-    std::vector<uint8_t> mb;
-    for (int k = 0; k < njobs; k++) {
-      const zipnn_stream* s = used[(size_t)k];
-      const uint64_t mbytes = (uint64_t)s->n_chunks * s->n_groups * kEntryBytes;
-      if (s->nbytes < kHdrBytes + mbytes) continue;  // malformed: the decoder reports it
+  DecodeGroup groups[kDecodeFamilies];
+  const int ngroups = group_decode_jobs(jobs, chunks, groups);
+  // stages from the chunk maps present now
+  std::vector<uint8_t> mb;
+  for (int k = 0; k < ngroups; k++) {
+    DecodeGroup& G = groups[k];
+    MapNeed nd;
+    const uint64_t dflt = G.shape.max_chunk * (uint64_t)G.shape.frac64 / 64 + 1024;
+    for (int i = G.first; i < G.first + G.count; i++) {
+      const Job& J = jobs[(size_t)i];
+      const uint64_t end = i + 1 < G.first + G.count ? jobs[(size_t)i + 1].chunk_begin : G.nchunks;
+      const uint32_t ng = (uint32_t)elem_size(J.dtype);
+      const uint64_t mbytes = (uint64_t)J.n_chunks * ng * kEntryBytes;
+      if (J.stream_bytes < kHdrBytes + mbytes) continue;  // malformed: the decoder reports it
       mb.resize((size_t)mbytes);
-      if (mbytes && cudaMemcpy(mb.data(), static_cast<const uint8_t*>(s->data) + kHdrBytes,
-                               (size_t)mbytes, cudaMemcpyDeviceToHost) != cudaSuccess)
+      if (mbytes && cudaMemcpy(mb.data(), J.src + kHdrBytes, (size_t)mbytes,
+                               cudaMemcpyDeviceToHost) != cudaSuccess)
         return ZIPNN_ECUDA;
-      const Job& J = jobs[(size_t)k];
-      const uint64_t n = k + 1 < njobs ? jobs[(size_t)k + 1].chunk_begin - J.chunk_begin
-                                       : chunk - J.chunk_begin;
-      add_map_need(mb.data() + (uint64_t)J.chunk0 * s->n_groups * kEntryBytes, (uint32_t)n,
-                   s->n_groups, w, dflt, &nd);
+      add_map_need(mb.data() + (uint64_t)J.chunk0 * ng * kEntryBytes, (uint32_t)(end - J.chunk_begin),
+                   ng, dflt, &nd);
     }
+    G.shape.stage_need = planned_stage(nd);
   }
   uint32_t* err = plan_err_word();
   if (!err) return ZIPNN_ECUDA;
@@ -208,19 +189,13 @@ static zipnn_status plan_decode_range(const zipnn_stream* streams, const void* c
   Job* d_jobs = static_cast<Job*>(p->dmem);
   auto* ticket = reinterpret_cast<unsigned long long*>(static_cast<uint8_t*>(p->dmem) + tbytes);
   e = cudaMemcpy(d_jobs, jobs.data(), sizeof(Job) * (size_t)njobs, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemset(ticket, 0, 2 * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMemset(ticket, 0, 2 * sizeof(unsigned long long) * kDecodeFamilies);
   if (e != cudaSuccess) return fail(p, e);
   zipnn_tuning tu;
   memset(&tu, 0, sizeof(tu));
   if (tuning) tu = *tuning;
-  const int uni = uniform < 0 ? -1 : uniform;
-  uint32_t common_lanes = jobs[0].lanes;
-  for (const Job& J : jobs)
-    if (J.lanes != common_lanes) common_lanes = 0;
   e = capture(p, [&](cudaStream_t cs) {
-    return launch_decode_ex(d_jobs, nullptr, njobs, chunk, max_groups, &tu, err, ticket, cs, uni,
-                            max_chunk, lanes256, frac64, has_delta, nd.general,
-                            planned_stage(nd), common_lanes);
+    return launch_decode_groups(d_jobs, groups, ngroups, &tu, err, ticket, cs);
   });
   if (e != cudaSuccess) return fail(p, e);
   *out = p;
@@ -373,12 +348,35 @@ zipnn_status zipnn_plan_load(const zipnn_stream* streams, const void* const* h_c
   }
   const int nseg = (int)seg_first.size();
   seg_first.push_back(count);
-  // chunk numbering restarts in every segment (each has its own table and ticket)
+  // each segment's jobs, grouped by dtype family (chunk numbering restarts in
+  // every group: each has its own part of the table and its own tickets), and
+  // their stages from the host copies' chunk maps
+  struct Segment {
+    DecodeGroup groups[kDecodeFamilies];
+    int n = 0;
+  };
+  std::vector<Segment> segs((size_t)nseg);
   for (int k = 0; k < nseg; k++) {
-    uint64_t ch = 0;
-    for (int i = seg_first[k]; i < seg_first[k + 1]; i++) {
-      jobs[i].chunk_begin = ch;
-      ch += jobs[i].n_chunks;
+    const int a = seg_first[k], b = seg_first[k + 1];
+    Segment& sg = segs[(size_t)k];
+    std::vector<Job> part(jobs.begin() + a, jobs.begin() + b);
+    std::vector<uint64_t> chunks;
+    for (const Job& J : part) chunks.push_back(J.n_chunks);
+    sg.n = group_decode_jobs(part, chunks, sg.groups);
+    std::copy(part.begin(), part.end(), jobs.begin() + a);
+    for (int f = 0; f < sg.n; f++) {
+      DecodeGroup& G = sg.groups[f];
+      MapNeed nd;
+      const uint64_t dflt = G.shape.max_chunk * (uint64_t)G.shape.frac64 / 64 + 1024;
+      for (int i = a; i < b; i++) {
+        const zipnn_stream* s = &streams[i];
+        if (dtype_family(s->dtype) != G.shape.family) continue;
+        const uint64_t mbytes = (uint64_t)s->n_chunks * s->n_groups * kEntryBytes;
+        if (s->nbytes < kHdrBytes + mbytes) continue;
+        add_map_need(static_cast<const uint8_t*>(h_containers[i]) + kHdrBytes, s->n_chunks,
+                     s->n_groups, dflt, &nd);
+      }
+      G.shape.stage_need = planned_stage(nd);
     }
   }
   uint32_t* err = plan_err_word();
@@ -388,7 +386,8 @@ zipnn_status zipnn_plan_load(const zipnn_stream* streams, const void* const* h_c
   p->count = count;
   cudaGetDevice(&p->device);
   const size_t tbytes = align_up(sizeof(Job) * (size_t)count, 256);
-  const size_t kbytes = align_up(2 * sizeof(unsigned long long) * (size_t)nseg, 256);
+  const size_t kbytes =
+      align_up(2 * sizeof(unsigned long long) * kDecodeFamilies * (size_t)nseg, 256);
   cudaError_t e = cudaMalloc(&p->dmem, tbytes + kbytes);
   if (e != cudaSuccess) return fail(p, e);
   Job* d_jobs = static_cast<Job*>(p->dmem);
@@ -412,32 +411,6 @@ zipnn_status zipnn_plan_load(const zipnn_stream* streams, const void* const* h_c
     if (r == cudaSuccess) r = cudaStreamWaitEvent(sc, evs[(size_t)nseg], 0);
     for (int k = 0; k < nseg && r == cudaSuccess; k++) {
       const int a = seg_first[k], b = seg_first[k + 1];
-      uint64_t nch = 0, max_chunk = 0;
-      int max_groups = 1, uniform = jobs[a].dtype;
-      bool lanes256 = true, has_delta = false;
-      int frac64 = 0;
-      for (int i = a; i < b; i++) {
-        if (stage_frac64(jobs[i].dtype, jobs[i].flags) > frac64)
-          frac64 = stage_frac64(jobs[i].dtype, jobs[i].flags);
-        if (jobs[i].chunk_bytes > max_chunk) max_chunk = jobs[i].chunk_bytes;
-      }
-      // stage and kernel variant from the host copies' chunk maps
-      MapNeed nd;
-      const uint64_t dflt = max_chunk * (uint64_t)frac64 / 64 + 1024;
-      for (int i = a; i < b; i++) {
-        const zipnn_stream* s = &streams[i];
-        const uint64_t mbytes = (uint64_t)s->n_chunks * s->n_groups * kEntryBytes;
-        if (s->nbytes < kHdrBytes + mbytes) continue;
-        add_map_need(static_cast<const uint8_t*>(h_containers[i]) + kHdrBytes, s->n_chunks,
-                     s->n_groups, plan_lut_bits(&tu), dflt, &nd);
-      }
-      for (int i = a; i < b; i++) {
-        if (jobs[i].flags & ZIPNN_FLAG_DELTA) has_delta = true;
-        nch += jobs[i].n_chunks;
-        if (jobs[i].dtype != uniform) uniform = -1;
-        if ((int)streams[i].n_groups > max_groups) max_groups = (int)streams[i].n_groups;
-        if (jobs[i].lanes % 256) lanes256 = false;
-      }
       // one copy per run of containers that sit back to back in both host and
       // device memory (each copy costs the copy engine a few microseconds of
       // setup); exact adjacency only, so no byte outside a container is written
@@ -452,13 +425,10 @@ zipnn_status zipnn_plan_load(const zipnn_stream* streams, const void* const* h_c
       }
       if (r == cudaSuccess) r = cudaEventRecord(evs[(size_t)k], sc);
       if (r == cudaSuccess) r = cudaStreamWaitEvent(cs, evs[(size_t)k], 0);
-      uint32_t common_lanes = jobs[a].lanes;
-      for (int i = a; i < b; i++)
-        if (jobs[i].lanes != common_lanes) common_lanes = 0;
+      const Segment& sg = segs[(size_t)k];
       if (r == cudaSuccess)
-        r = launch_decode_ex(d_jobs + a, nullptr, b - a, nch, max_groups, &tu, err,
-                             tickets + 2 * k, cs, uniform, max_chunk, lanes256, frac64,
-                             has_delta, nd.general, planned_stage(nd), common_lanes);
+        r = launch_decode_groups(d_jobs + a, sg.groups, sg.n, &tu, err,
+                                 tickets + 2 * kDecodeFamilies * k, cs);
     }
     // the last wait above joined the copy stream back into the capture stream
     return r;

@@ -27,23 +27,28 @@ enum Mode : uint32_t { kRaw = 0, kHuff = 1, kZero = 2, kConst = 3, kSparse = 4 }
 __host__ __device__ inline int elem_size(int dtype) {
   return dtype == ZIPNN_FP32 ? 4 : (dtype == ZIPNN_U8 ? 1 : 2);
 }
+// FP16 has BF16's byte groups (the same 16-bit permutation): the decoder's
+// kernels serve both.
+__host__ __device__ inline int dtype_family(int dtype) {
+  return dtype == ZIPNN_FP16 ? ZIPNN_BF16 : dtype;
+}
 __host__ __device__ inline uint64_t align_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
 
 // Decoder stage sizing: the Huffman payload bytes of one chunk to provision
 // for, in 64ths of the chunk.  Model weights: a BF16 exponent group codes to
 // about a third of its half of the chunk (11/64 with margin), an FP16 one (5
 // exponent + 3 fraction bits) to about 70% (24/64), an FP32 one to about a
-// third of its quarter (8/64); U8 streams are unknown (32/64); a BF16 / FP32
-// delta codes two groups, and the stage also holds the second group's table
-// (20/64).  Chunks whose payloads exceed the stage are decoded from global
-// memory instead.
+// third of its quarter (8/64).  A BF16 / FP32 delta codes two groups, to about
+// 0.14 of the chunk between checkpoints (9/64: with two tables, three 256-thread
+// CTAs per SM at 256 KiB).  U8 streams are not staged.  Payloads that exceed the
+// stage are decoded in slices of their sub-streams.
 inline int stage_frac64(int dtype, uint32_t flags) {
   const bool delta = (flags & 1u) != 0;
   switch (dtype) {
-    case 0: return delta ? 20 : 11;
+    case 0: return delta ? 9 : 11;
     case 1: return 24;
-    case 2: return delta ? 20 : 8;
-    default: return 32;
+    case 2: return delta ? 9 : 8;
+    default: return 8;
   }
 }
 

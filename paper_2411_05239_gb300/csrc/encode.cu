@@ -1046,16 +1046,23 @@ __device__ __forceinline__ uint32_t len4(uint32_t cb, uint32_t w) {
          (code_of(cb, w, 3) >> 16);
 }
 
+// Whole vectors of unit (t, k): part k of sub-stream t, of at most per vectors
+// (v = t + (k per + i) T), in a chunk of nfull whole vectors.
+__device__ __forceinline__ uint32_t unit_vectors(uint32_t t, uint32_t k, uint32_t T, uint32_t per,
+                                                 uint32_t nfull) {
+  const uint32_t cnt = nfull > t ? gdiv(nfull - t + T - 1u, T) : 0u, i0 = k * per;
+  return cnt > i0 ? min(per, cnt - i0) : 0u;
+}
+
 // Pass A for the dominant chunk layout: group 0 Huffman (slot-encoded), every
-// other group raw, zero or constant (bit g of raw set for raw groups), a whole
-// chunk whose vectors split evenly over the T sub-streams and R parts (per
-// vectors per unit).  No tails: per vector one 16-B load (two in flight, the
-// line requested from L2 eight vectors earlier), the
-// split, V/4 joined code appends into the unit's slot and one store per raw
-// group.
+// other group raw, zero or constant (bit g of raw set for raw groups), per
+// vectors per unit at most.  Per vector one 16-B load (two in flight, the line
+// requested from L2 eight vectors earlier), the split, V/4 joined code appends
+// into the unit's slot and one store per raw group.  (The partial last vector of
+// a ragged chunk is appended afterwards, see pack_partial.)
 template <int DT>
-__device__ __forceinline__ void pack_fast_a(const uint8_t* src, const uint8_t* base, uint32_t T,
-                                            uint32_t R, uint32_t per, uint32_t* slots,
+__device__ __forceinline__ void pack_fast_a(const uint8_t* src, const uint8_t* base, uint32_t nfull,
+                                            uint32_t T, uint32_t R, uint32_t chunk_per, uint32_t* slots,
                                             uint32_t slot_cap, PackSmem& S, uint8_t* out,
                                             uint64_t P, uint32_t raw) {
   constexpr int G = PTraits<DT>::G, V = PTraits<DT>::V;
@@ -1084,13 +1091,16 @@ __device__ __forceinline__ void pack_fast_a(const uint8_t* src, const uint8_t* b
     sw.wi = 0;
     sw.cap = slot_cap;
     sw.bits = 0;
-    uint32_t v = t + k * per * T;
+    const uint32_t per = unit_vectors(t, k, T, chunk_per, nfull);
+    uint32_t v = t + k * chunk_per * T;
     constexpr uint32_t D = 2;
     for (uint32_t i = D; i < kPrefetchAhead && i < per; i++) {
       prefetch_l2(s4 + v + i * T);
       if (base) prefetch_l2(b4 + v + i * T);
     }
-    uint4 a0 = ld(v), a1 = per > 1 ? ld(v + T) : make_uint4(0, 0, 0, 0);
+    uint4 a0 = make_uint4(0, 0, 0, 0), a1 = a0;
+    if (per > 0) a0 = ld(v);
+    if (per > 1) a1 = ld(v + T);
     auto one = [&](uint4& a, uint32_t i) {
       uint32_t g4[4][4];
       split_vec(DT, a, g4);
@@ -1246,7 +1256,9 @@ __device__ __forceinline__ uint32_t pair_unit(const uint4* __restrict__ s4,
     v += T;
   };
   for (uint32_t i = 2; i < kPrefetchAhead && i < per; i++) pf(v + i * T);
-  uint4 a0 = ld(v), a1 = per > 1 ? ld(v + T) : make_uint4(0, 0, 0, 0);
+  uint4 a0 = make_uint4(0, 0, 0, 0), a1 = a0;
+  if (per > 0) a0 = ld(v);
+  if (per > 1) a1 = ld(v + T);
   uint32_t i = 0;
   for (; i + kPrefetchAhead + 1 < per; i += 2) {
     one(a0, true, true);
@@ -1321,7 +1333,9 @@ __device__ __forceinline__ uint32_t pair_unit32(const uint4* __restrict__ s4,
     v += T;
   };
   for (uint32_t i = 2; i < kPrefetchAhead && i < per; i++) pf(v + i * T);
-  uint4 a0 = ld(v), a1 = per > 1 ? ld(v + T) : make_uint4(0, 0, 0, 0);
+  uint4 a0 = make_uint4(0, 0, 0, 0), a1 = a0;
+  if (per > 0) a0 = ld(v);
+  if (per > 1) a1 = ld(v + T);
   uint32_t i = 0;
   for (; i + kPrefetchAhead + 1 < per; i += 2) {
     one(a0, true, true);
@@ -1336,8 +1350,8 @@ __device__ __forceinline__ uint32_t pair_unit32(const uint4* __restrict__ s4,
 }
 
 template <int DT>
-__device__ __forceinline__ void pack_pair_a(const uint8_t* src, const uint8_t* base, uint32_t T,
-                                            uint32_t R, uint32_t per, uint32_t* slots,
+__device__ __forceinline__ void pack_pair_a(const uint8_t* src, const uint8_t* base, uint32_t nfull,
+                                            uint32_t T, uint32_t R, uint32_t per, uint32_t* slots,
                                             uint32_t slot_cap, PackSmem& S, uint8_t* out,
                                             uint64_t P, uint32_t raw) {
   static_assert(DT == ZIPNN_BF16 || DT == ZIPNN_FP16 || DT == ZIPNN_FP32,
@@ -1355,9 +1369,9 @@ __device__ __forceinline__ void pack_pair_a(const uint8_t* src, const uint8_t* b
     for (uint32_t u = tid; u < units; u += nthr) {
       const uint32_t t = gmod(u, T), k = gdiv(u, T), ui = t * R + k;
       const uint32_t sa0 = smem_u32(slots) + 4u * ui * slot_cap, slast = sa0 + 4u * (slot_cap - 1);
-      const uint32_t v = t + k * per * T;
-      const uint32_t bits = base ? pair_unit32<true>(s4, b4, rawp, v, T, per, pb16, sa0, slast)
-                                 : pair_unit32<false>(s4, b4, rawp, v, T, per, pb16, sa0, slast);
+      const uint32_t v = t + k * per * T, n = unit_vectors(t, k, T, per, nfull);
+      const uint32_t bits = base ? pair_unit32<true>(s4, b4, rawp, v, T, n, pb16, sa0, slast)
+                                 : pair_unit32<false>(s4, b4, rawp, v, T, n, pb16, sa0, slast);
       S.sbits[ui] = bits;
       S.part[0][ui] = bits;
     }
@@ -1371,16 +1385,57 @@ __device__ __forceinline__ void pack_pair_a(const uint8_t* src, const uint8_t* b
   for (uint32_t u = tid; u < units; u += nthr) {
     const uint32_t t = gmod(u, T), k = gdiv(u, T), ui = t * R + k;
     const uint32_t sa0 = smem_u32(slots) + 4u * ui * slot_cap, slast = sa0 + 4u * (slot_cap - 1);
-    const uint32_t v = t + k * per * T;
+    const uint32_t v = t + k * per * T, n = unit_vectors(t, k, T, per, nfull);
     uint32_t bits;
     if (base)
-      bits = rw ? pair_unit<true, true>(s4, b4, rawp, v, T, per, pb16, sa0, slast)
-                : pair_unit<true, false>(s4, b4, rawp, v, T, per, pb16, sa0, slast);
+      bits = rw ? pair_unit<true, true>(s4, b4, rawp, v, T, n, pb16, sa0, slast)
+                : pair_unit<true, false>(s4, b4, rawp, v, T, n, pb16, sa0, slast);
     else
-      bits = rw ? pair_unit<false, true>(s4, b4, rawp, v, T, per, pb16, sa0, slast)
-                : pair_unit<false, false>(s4, b4, rawp, v, T, per, pb16, sa0, slast);
+      bits = rw ? pair_unit<false, true>(s4, b4, rawp, v, T, n, pb16, sa0, slast)
+                : pair_unit<false, false>(s4, b4, rawp, v, T, n, pb16, sa0, slast);
     S.sbits[ui] = bits;
     S.part[0][ui] = bits;
+  }
+}
+
+// After pass A (fast): the partial last vector of a ragged chunk, by the thread
+// of the unit that it belongs to (the one after which it continues sub-stream
+// nfull mod T): its symbols appended to the unit's slot one by one, its raw
+// bytes (those past the chunk are the zeros of the payload's padding).
+template <int DT>
+__device__ __forceinline__ void pack_partial(const uint8_t* src, const uint8_t* base, uint32_t nb,
+                                             uint32_t T, uint32_t R, uint32_t per, uint32_t* slots,
+                                             uint32_t slot_cap, PackSmem& S, uint8_t* out,
+                                             uint64_t P, uint32_t raw) {
+  constexpr int G = PTraits<DT>::G, V = PTraits<DT>::V, ES = 16 / V;
+  const uint32_t nfull = nb / 16u, t = gmod(nfull, T), k = gdiv(gdiv(nfull, T), per);
+  if (threadIdx.x != gmod(k * T + t, blockDim.x)) return;
+  const uint32_t valid = (nb % 16u) / ES, ui = t * R + k;
+  const uint32_t slot = smem_u32(slots) + 4u * ui * slot_cap;
+  uint32_t g4[4][4];
+  split_vec(DT, load_vec(src, base, nfull, nb), g4);
+  SlotWriter sw;  // continued from the unit's bits
+  sw.slot = slot;
+  sw.bits = S.sbits[ui];
+  sw.nacc = sw.bits & 31u;
+  sw.wi = sw.bits >> 5;
+  sw.cap = slot_cap;
+  sw.acc = sw.nacc && sw.wi < slot_cap ? lds32v(slot + 4u * sw.wi) >> (32u - sw.nacc) : 0u;
+#pragma unroll
+  for (int q = 0; q < V; q++)
+    if (q < (int)valid) {
+      const uint32_t cl = code_of(smem_u32(S.codes[0]), g4[0][q >> 2], q & 3);
+      sw.put(cl & 0xFFFFu, cl >> 16);
+    }
+  sw.finish();
+  S.sbits[ui] = sw.bits;
+  S.part[0][ui] = sw.bits;
+#pragma unroll
+  for (int g = 1; g < G; g++) {
+    if (!(raw >> g & 1u)) continue;
+    uint8_t* p = out + P + S.off[g];
+    if (V == 8) reinterpret_cast<uint2*>(p)[nfull] = make_uint2(g4[g][0], g4[g][1]);
+    else reinterpret_cast<uint32_t*>(p)[nfull] = g4[g][0];
   }
 }
 
@@ -1560,9 +1615,7 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
   }
   if (!(slot_cap & 1u)) slot_cap--;
   const uint32_t slots1 = smem_u32(slots) + 4u * units * slot_cap;  // second group's slots
-  const bool fast_a = sg == 0 && huff == 1u && sparse == 0 && nb == J.chunk_bytes &&
-                      gmod((uint32_t)nvec, T) == 0 && gmod((uint32_t)nvt, R) == 0 &&
-                      T <= (uint32_t)nthr;
+  const bool fast_a = sg == 0 && huff == 1u && sparse == 0;
   bool pairs = false;
   if constexpr (DT == ZIPNN_BF16 || DT == ZIPNN_FP16 || DT == ZIPNN_FP32)
     pairs = fast_a && smem_u32(S.ptab) + 4096u <= 65536u && build_pair_table(S);
@@ -1572,10 +1625,12 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
   if (fast_a) {
     if constexpr (DT == ZIPNN_BF16 || DT == ZIPNN_FP16 || DT == ZIPNN_FP32) {
       if (pairs)
-        pack_pair_a<DT>(src, base, T, R, gdiv((uint32_t)nvt, R), slots, slot_cap, S, out, P, raw);
+        pack_pair_a<DT>(src, base, (uint32_t)nb / 16u, T, R, (uint32_t)per, slots, slot_cap, S, out, P, raw);
     }
     if (!pairs)
-      pack_fast_a<DT>(src, base, T, R, gdiv((uint32_t)nvt, R), slots, slot_cap, S, out, P, raw);
+      pack_fast_a<DT>(src, base, (uint32_t)nb / 16u, T, R, (uint32_t)per, slots, slot_cap, S, out, P, raw);
+    if (nb % 16)
+      pack_partial<DT>(src, base, (uint32_t)nb, T, R, (uint32_t)per, slots, slot_cap, S, out, P, raw);
   }
   for (uint32_t u = fast_a ? units : tid; u < units; u += nthr) {
     const uint32_t t = gmod(u, T), k = gdiv(u, T);

@@ -434,20 +434,75 @@ __device__ __forceinline__ int lower_bound_u32(const uint32_t* a, int n, uint32_
 }
 
 // Shannon bound: any prefix code spends >= sum c log2(n / c) bits on counts c
-// summing to n.  True when even that many bits (plus `fixed` bytes) cannot
-// qualify against the raw size m, or, with have_best, cannot beat `best`.
-__device__ bool bound_rules_out(const uint32_t cnt[8], uint32_t n, uint64_t fixed, uint32_t m,
-                                bool have_best, uint64_t best) {
+// summing to n.  A lower bound of the size of such a code's payload with
+// `fixed` bytes before the bitstream.
+__device__ uint64_t least_size(const uint32_t cnt[8], uint32_t n, uint64_t fixed) {
   float part = 0.f;
   const float lm = log2f((float)n);
+#pragma unroll
   for (int k = 0; k < 8; k++)
     if (cnt[k]) part += (float)cnt[k] * (lm - log2f((float)cnt[k]));
   for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
   const float lower = part * (1.0f - 1e-4f) - 64.0f;
-  if (!(lower > 0.f)) return false;
-  const uint64_t lb_bits = (uint64_t)lower;
-  const uint64_t lb_size = fixed + 4ull * ((lb_bits + 31) / 32);
-  return lb_size + (m >> 6) >= m || (have_best && lb_size >= best);
+  if (!(lower > 0.f)) return fixed;
+  return fixed + 4ull * (((uint64_t)lower + 31) / 32);
+}
+
+// Code lengths for 2 <= nz <= 32 non-zero symbols, in registers: lane i holds
+// the i-th non-zero symbol's key (count << 8 | 255 - symbol), later the i-th
+// smallest leaf.  A list of the package-merge lies two items to a lane, so its
+// packages are the lanes' sums; leaves and packages find their places in the
+// merged list by counting each other with shuffles (5 or 6 dependent steps),
+// and the list takes its new order through shared memory.  (The exponent groups
+// of model weights: this latency, not throughput, is what a small call waits
+// for; the lists in shared memory took 11 levels of about 1.5 us.)
+__device__ void pm_lengths_small(BuildSmem& S, uint32_t key, uint32_t nz, int lane) {
+  const int n = (int)nz;
+  uint32_t r = 0;
+#pragma unroll
+  for (int q = 0; q < 32; q++) r += __shfl_sync(0xffffffffu, key, q) < key;
+  if (lane < n) S.lst[0][r] = key;
+  __syncwarp();
+  const uint32_t leaf = lane < n ? S.lst[0][lane] : 0xFFFFFFFFu;
+  const uint32_t w = lane < n ? leaf >> 8 : 0xFFFFFFFFu;
+  uint32_t a0 = __shfl_sync(0xffffffffu, w, 2 * lane & 31), a1 = __shfl_sync(0xffffffffu, w, (2 * lane + 1) & 31);
+  int sp = n;
+  uint32_t pos[kMaxLen];  // this leaf's place in each list
+#pragma unroll
+  for (int lvl = 1; lvl < kMaxLen; lvl++) {
+    const int np = sp >> 1;
+    const uint32_t pk = lane < np ? a0 + a1 : 0xFFFFFFFFu;
+    uint32_t cp = 0, cl = 0;  // packages below this leaf, leaves up to this package
+#pragma unroll
+    for (int st = 16; st; st >>= 1) {
+      const uint32_t x = __shfl_sync(0xffffffffu, pk, (int)cp + st - 1);
+      const uint32_t y = __shfl_sync(0xffffffffu, w, (int)cl + st - 1);
+      if (x < w) cp += st;
+      if (y <= pk) cl += st;
+    }
+    if (__shfl_sync(0xffffffffu, w, (int)cl) <= pk) cl++;  // (all 32 leaves)
+    uint32_t* to = S.lst[lvl & 1];
+    pos[lvl] = lane < n ? lane + cp : 0xFFFFu;
+    if (lane < n) to[pos[lvl]] = w;
+    if (lane < np) to[lane + cl] = pk;
+    __syncwarp();
+    sp = n + np;
+    a0 = to[2 * lane];
+    a1 = to[2 * lane + 1];
+  }
+  // selection, from the last list down: the first `take` items of a list hold
+  // a leaves and take - a packages, which select twice as many of the next
+  int take = 2 * (n - 1);
+  uint32_t len = 0;
+#pragma unroll
+  for (int lvl = kMaxLen - 1; lvl >= 1; lvl--) {
+    const int leaves = __popc(__ballot_sync(0xffffffffu, (int)pos[lvl] < take));
+    len += lane < leaves;
+    take = 2 * (take - leaves);
+  }
+  len += lane < take;  // list 0 holds leaves only
+  if (lane < n) S.lens[255u - (leaf & 0xFFu)] = (uint8_t)len;
+  __syncwarp();
 }
 
 // Code lengths limited to kMaxLen bits for the counts cnt[k] of symbols
@@ -469,6 +524,12 @@ __device__ void pm_lengths(BuildSmem& S, const uint32_t cnt[8], uint32_t nz, int
     }
   }
   __syncwarp();
+  if (nz <= 32) {
+    for (int k = 0; k < 8; k++)
+      if (!cnt[k]) S.lens[lane + 32 * k] = 0;
+    pm_lengths_small(S, lane < (int)nz ? S.keys[lane] : 0xFFFFFFFFu, nz, lane);
+    return;
+  }
   if (nz <= 96) {
     for (uint32_t i = lane; i < nz; i += 32) {
       const uint32_t key = S.keys[i];
@@ -651,73 +712,89 @@ __device__ void build_gc(const uint32_t* hist256, uint32_t zs, uint32_t m, uint3
 
   const uint32_t V = 16u / (uint32_t)es, nv = (m + V - 1) / V;
 
-  // HUFF candidate: a code for all m symbols (skipped when the Shannon bound
-  // already shows it cannot qualify)
-  const uint32_t h = (uint32_t)align_up(12 + nz, 4);
-  const uint64_t fixed = (uint64_t)h + 4ull * (T - 1);
-  bool huff_ok = false;
-  uint64_t hsize = 0;
-  uint8_t lenH[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  if (!bound_rules_out(cnt, m, fixed, m, false, 0)) {
-    pm_lengths(S, cnt, nz, lane);
-    uint32_t bits = 0;
+  // Two candidates: HUFF, a code for all m symbols; SPARSE, a code for the
+  // symbols outside all-zero vectors (the zeros of those vectors leave the
+  // histogram) plus a bitmap of the vectors.  A code is built only while the
+  // Shannon bound does not show that its candidate cannot qualify or cannot
+  // win, and the one with the smaller bound first, which mostly settles it.
+  const uint64_t fixed = align_up(12 + nz, 4) + 4ull * (T - 1);
+  uint32_t cnt2[8];
+  uint32_t nz2 = 0;
+#pragma unroll
+  for (int k = 0; k < 8; k++) cnt2[k] = cnt[k];
+  if (lane == 0) cnt2[0] -= zs;  // symbol 0 is lane 0, k = 0
+  if (zs > 0)
+    for (int k = 0; k < 8; k++) nz2 += __popc(__ballot_sync(0xffffffffu, cnt2[k] > 0));
+  const uint64_t fixed2 = align_up(12 + nz2, 4) + 4ull * ((nv + 31) / 32) + 4ull * (T - 1);
+  const uint64_t hleast = least_size(cnt, m, fixed);
+  const uint64_t sleast = nz2 >= 2 ? least_size(cnt2, m - zs, fixed2) : ~0ull >> 1;
+  // (SPARSE is taken only when strictly smaller than a qualifying HUFF)
+  res.mode = kRaw;
+  res.size = m;
+  uint32_t mylen[8];
+#pragma unroll
+  for (int k = 0; k < 8; k++) mylen[k] = 0;
+#pragma unroll 1
+  for (int turn = 0; turn < 2; turn++) {
+    const bool sp = (sleast < hleast) == (turn == 0);  // SPARSE's turn
+    const uint64_t least = sp ? sleast : hleast;
+    if (least + (m >> 6) >= m) continue;
+    const bool have = res.mode != kRaw;  // the other one qualifies
+    if (have && (sp ? least >= res.size : least > res.size)) continue;
+    uint32_t c[8];
+#pragma unroll
+    for (int k = 0; k < 8; k++) c[k] = sp ? cnt2[k] : cnt[k];
+    pm_lengths(S, c, sp ? nz2 : nz, lane);
+    uint32_t bits = 0, len[8];
+#pragma unroll
     for (int k = 0; k < 8; k++) {
-      lenH[k] = S.lens[lane + 32 * k];
-      bits += cnt[k] * lenH[k];
+      len[k] = S.lens[lane + 32 * k];
+      bits += c[k] * len[k];
     }
     for (int o = 16; o; o >>= 1) bits += __shfl_xor_sync(0xffffffffu, bits, o);
-    hsize = fixed + 4ull * ((bits + 31) / 32);
-    huff_ok = hsize + (m >> 6) < m;
+    const uint64_t size = (sp ? fixed2 : fixed) + 4ull * ((bits + 31) / 32);
+    if (size + (m >> 6) < m && !(have && (sp ? size >= res.size : size > res.size))) {
+      res.mode = sp ? kSparse : kHuff;
+      res.size = (uint32_t)size;
+      res.nz = sp ? nz2 : nz;
+#pragma unroll
+      for (int k = 0; k < 8; k++) mylen[k] = len[k];
+    }
     __syncwarp();
   }
-
-  // SPARSE candidate: a code for the symbols outside all-zero vectors (the
-  // zeros of those vectors leave the histogram) plus a bitmap of the vectors
-  bool sparse_ok = false;
-  uint64_t ssize = 0;
-  uint32_t nz2 = 0;
-  uint8_t lenS[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  if (zs > 0) {
-    uint32_t cnt2[8];
-    for (int k = 0; k < 8; k++) cnt2[k] = cnt[k];
-    if (lane == 0) cnt2[0] -= zs;                    // symbol 0 is lane 0, k = 0
-    for (int k = 0; k < 8; k++) nz2 += __popc(__ballot_sync(0xffffffffu, cnt2[k] > 0));
-    if (nz2 >= 2) {
-      const uint64_t fixed2 = align_up(12 + nz2, 4) + 4ull * ((nv + 31) / 32) + 4ull * (T - 1);
-      if (!bound_rules_out(cnt2, m - zs, fixed2, m, huff_ok, hsize)) {
-        pm_lengths(S, cnt2, nz2, lane);
-        uint32_t bits2 = 0;
-        for (int k = 0; k < 8; k++) {
-          lenS[k] = S.lens[lane + 32 * k];
-          bits2 += cnt2[k] * lenS[k];
-        }
-        for (int o = 16; o; o >>= 1) bits2 += __shfl_xor_sync(0xffffffffu, bits2, o);
-        ssize = fixed2 + 4ull * ((bits2 + 31) / 32);
-        sparse_ok = ssize + (m >> 6) < m;
-        __syncwarp();
-      }
-    }
-  }
-
-  // --- mode decision (SPARSE only when strictly smaller than a qualifying HUFF)
-  uint8_t mylen[8];
-  if (sparse_ok && (!huff_ok || ssize < hsize)) {
-    res.mode = kSparse;
-    res.size = (uint32_t)ssize;
-    res.nz = nz2;
-    for (int k = 0; k < 8; k++) mylen[k] = lenS[k];
-  } else if (huff_ok) {
-    res.mode = kHuff;
-    res.size = (uint32_t)hsize;
-    for (int k = 0; k < 8; k++) mylen[k] = lenH[k];
-  } else {
-    res.mode = kRaw;
-    res.size = m;
+  if (res.mode == kRaw) {
     if (lane == 0) *meta_out = res;
     return;
   }
 
   // --- canonical codes (RFC 1951 Sec. 3.2.2) and the table bytes
+  if (res.nz <= 32) {
+    // lane i takes the i-th symbol that has a code: one ballot per length
+    uint32_t basek = 0;
+    for (int k = 0; k < 8; k++) {
+      const uint32_t b = __ballot_sync(0xffffffffu, mylen[k] > 0);
+      if (mylen[k])
+        S.keys[basek + __popc(b & ((1u << lane) - 1u))] = ((uint32_t)mylen[k] << 8) | (uint32_t)(lane + 32 * k);
+      basek += __popc(b);
+    }
+    __syncwarp();
+    const uint32_t key = lane < (int)res.nz ? S.keys[lane] : 0u, len = key >> 8, sym = key & 0xFFu;
+    uint32_t code = 0, before = 0, prev = 0;
+    for (int l = 1; l <= kMaxLen; l++) {
+      const uint32_t b = __ballot_sync(0xffffffffu, (int)len == l);
+      code = (code + prev) << 1;
+      if ((int)len == l) {
+        const uint32_t r = __popc(b & ((1u << lane) - 1u));
+        mycodes[sym] = (len << 16) | (code + r);
+        tab[12 + before + r] = (uint8_t)sym;
+      }
+      prev = __popc(b);
+      before += prev;
+      if (lane == 0) tab[l - 1] = (uint8_t)prev;
+    }
+    if (lane == 0) *meta_out = res;
+    return;
+  }
   uint32_t count[kMaxLen + 1];
   for (int l = 0; l <= kMaxLen; l++) count[l] = 0;
   for (int l = 1; l <= kMaxLen; l++)
@@ -743,7 +820,7 @@ __device__ void build_gc(const uint32_t* hist256, uint32_t zs, uint32_t m, uint3
 }
 
 
-__global__ void __launch_bounds__(kBuildWarps * 32)
+__global__ void __launch_bounds__(kBuildWarps * 32, 6)
 k_build(JobRef jr, uint64_t ngc_total, const uint32_t* __restrict__ hist,
         const uint32_t* __restrict__ zsyms, uint32_t* __restrict__ codes,
         uint8_t* __restrict__ tabs, GcMeta* __restrict__ meta) {

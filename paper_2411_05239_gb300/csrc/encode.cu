@@ -964,6 +964,7 @@ struct PackSmem {
   uint32_t hsz[4];    // table + start-offset bytes before the bitstream
   uint32_t sbits[kPackMaxUnits];  // bits of each unit of the slot-staged group
   uint32_t ptab[1024];  // pair table of the 16-bit pass A (pack_pair_a)
+  uint32_t etab[256];   // group 1's code as table entries (pack_coded_a)
 };
 
 // Exclusive scan of a[0..n) in place (block-wide), the total into a[n];
@@ -1475,44 +1476,176 @@ __device__ __forceinline__ void pack_pair_a(const uint8_t* src, const uint8_t* b
   }
 }
 
+// Pass A of 16-bit delta chunks with both groups coded (HUFF, or SPARSE: SP0,
+// SP1) and staged, whose XOR-ed exponents have distinct residues mod 32.
+// Entries of the tables are (code << 6) | length, of one symbol (etab, group 1)
+// or two (ptab, group 0); two of etab's are joined into one of two symbols, and
+// four symbols are appended to a slot at a time.  In SPARSE groups a ballot
+// gathers the vectors' bitmap bits and all-zero vectors append nothing.
+struct SlotTail {  // a slot being written: next word, pending bits (the low nb of hi:lo)
+  uint32_t sa, lo, hi, nb;
+  __device__ __forceinline__ void put(uint32_t v, uint32_t n, uint32_t slast) {  // n <= 32 bits
+    hi = __funnelshift_lc(lo, hi, n);
+    lo = __funnelshift_lc(0u, lo, n) | v;
+    nb += n;
+    sts32(min(sa, slast), __funnelshift_r(lo, hi, nb - 32u));  // the word if nb >= 32
+    const bool full = nb >= 32;
+    sa += full ? 4u : 0u;
+    nb -= full ? 32u : 0u;
+  }
+  // the eight symbols of four entries of two
+  __device__ __forceinline__ void put8(uint32_t e0, uint32_t e1, uint32_t e2, uint32_t e3,
+                                       uint32_t slast) {
+    const uint32_t n0 = (e0 + e1) & 63u, n1 = (e2 + e3) & 63u;
+    if (max(n0, n1) <= 32u) {
+      put(__funnelshift_l(0u, e0 >> 6, e1) | (e1 >> 6), n0, slast);
+      put(__funnelshift_l(0u, e2 >> 6, e3) | (e3 >> 6), n1, slast);
+    } else {
+      put(e0 >> 6, e0 & 63u, slast);
+      put(e1 >> 6, e1 & 63u, slast);
+      put(e2 >> 6, e2 & 63u, slast);
+      put(e3 >> 6, e3 & 63u, slast);
+    }
+  }
+  __device__ __forceinline__ uint32_t finish(uint32_t sa0, uint32_t slast) {  // the slot's bits
+    if (nb) sts32(min(sa, slast), lo << (32 - nb));
+    return (sa - sa0) * 8u + nb;
+  }
+};
+// Entry of two symbols from two entries of one.
+__device__ __forceinline__ uint32_t join_entries(uint32_t a, uint32_t b) {
+  return __funnelshift_l(0u, a & ~63u, b) + b + (a & 63u);
+}
+
+template <bool SP0, bool SP1>
+__device__ __forceinline__ void pack_coded_a(const uint4* __restrict__ s4, const uint4* __restrict__ b4,
+                                             uint32_t nfull, uint32_t T, uint32_t R, uint32_t per,
+                                             uint32_t slots, uint32_t slot_cap, uint32_t slots1,
+                                             uint32_t slot_cap1, PackSmem& S, uint32_t* bmap0,
+                                             uint32_t* bmap1) {
+  const uint32_t tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31u;
+  const uint32_t pb16 = smem_u32(S.ptab) << 16, et = smem_u32(S.etab);
+  auto ld = [&](uint32_t v) -> uint4 {
+    uint4 a = __ldg(s4 + v);
+    const uint4 b = __ldg(b4 + v);
+    a.x ^= b.x; a.y ^= b.y; a.z ^= b.z; a.w ^= b.w;
+    return a;
+  };
+  auto pf = [&](uint32_t v) {
+    prefetch_l2(s4 + v);
+    prefetch_l2(b4 + v);
+  };
+  auto entry0 = [&](uint32_t x) -> uint32_t {  // group 0's entry of the element pair x
+    return lds32(((x & 0x0F800F80u) * 0x801u + pb16) >> 16);
+  };
+  auto entry1 = [&](uint32_t w, int k) -> uint32_t {  // group 1's entry of bytes k, k + 1 of w
+    return join_entries(lds32(et + 4u * __byte_perm(w, 0, 0x4440 + k)),
+                        lds32(et + 4u * __byte_perm(w, 0, 0x4440 + k + 1)));
+  };
+  // lanes of a warp hold consecutive vectors from a multiple of 32: where they
+  // also run equally long (whole chunks), one ballot is a bitmap word
+  const bool lockstep = gmod(nfull, T * per) == 0;
+  auto mark = [&](uint32_t* bm, uint32_t v, bool any) {
+    if (lockstep) {
+      const uint32_t word = __ballot_sync(0xffffffffu, any);
+      if (lane == 0) bm[v >> 5] = word;
+    } else if (any) {
+      atomicOr(&bm[v >> 5], 1u << (v & 31));
+    }
+  };
+  for (uint32_t u = tid; u < T * R; u += nthr) {
+    const uint32_t t = gmod(u, T), k = gdiv(u, T), ui = t * R + k;
+    const uint32_t sa0 = slots + 4u * ui * slot_cap, last0 = sa0 + 4u * (slot_cap - 1);
+    const uint32_t sa1 = slots1 + 4u * ui * slot_cap1, last1 = sa1 + 4u * (slot_cap1 - 1);
+    SlotTail w0 = {sa0, 0, 0, 0}, w1 = {sa1, 0, 0, 0};
+    uint32_t v = t + k * per * T;
+    const uint32_t n = unit_vectors(t, k, T, per, nfull);
+    for (uint32_t i = 2; i < kPrefetchAhead && i < n; i++) pf(v + i * T);
+    uint4 a0 = make_uint4(0, 0, 0, 0), a1 = a0;
+    if (n > 0) a0 = ld(v);
+    if (n > 1) a1 = ld(v + T);
+    auto one = [&](uint4& a, bool LD, bool PF) {
+      const uint4 x = a;
+      if (LD) a = ld(v + 2 * T);
+      if (PF) pf(v + kPrefetchAhead * T);
+      const uint32_t any = x.x | x.y | x.z | x.w;
+      const bool live0 = !SP0 || (any & 0x7F807F80u) != 0, live1 = !SP1 || (any & 0x807F807Fu) != 0;
+      if (SP0) mark(bmap0, v, live0);
+      if (SP1) mark(bmap1, v, live1);
+      if (live0) w0.put8(entry0(x.x), entry0(x.y), entry0(x.z), entry0(x.w), last0);
+      if (live1) {
+        uint32_t e, r0, r1;
+        split16(x.x, x.y, e, r0);
+        split16(x.z, x.w, e, r1);
+        w1.put8(entry1(r0, 0), entry1(r0, 2), entry1(r1, 0), entry1(r1, 2), last1);
+      }
+      v += T;
+    };
+    uint32_t i = 0;
+    for (; i + kPrefetchAhead + 1 < n; i += 2) {
+      one(a0, true, true);
+      one(a1, true, true);
+    }
+    for (; i < n; i += 2) {
+      one(a0, i + 2 < n, i + kPrefetchAhead < n);
+      if (i + 1 < n) one(a1, i + 3 < n, i + 1 + kPrefetchAhead < n);
+    }
+    const uint32_t bits0 = w0.finish(sa0, last0);
+    S.sbits[ui] = bits0;
+    S.part[0][ui] = bits0;
+    S.part[1][ui] = w1.finish(sa1, last1);
+  }
+}
+
 // After pass A (fast): the partial last vector of a ragged chunk, by the thread
 // of the unit that it belongs to (the one after which it continues sub-stream
-// nfull mod T): its symbols appended to the unit's slot one by one, its raw
-// bytes (those past the chunk are the zeros of the payload's padding).
+// nfull mod T): its symbols of group 0 (and, staged at slots1, of group 1)
+// appended to the unit's slots one by one, its raw bytes (those past the chunk
+// are the zeros of the payload's padding), its bitmap bits.
 template <int DT>
 __device__ __forceinline__ void pack_partial(const uint8_t* src, const uint8_t* base, uint32_t nb,
-                                             uint32_t T, uint32_t R, uint32_t per, uint32_t* slots,
-                                             uint32_t slot_cap, PackSmem& S, uint8_t* out,
-                                             uint64_t P, uint32_t raw) {
+                                             uint32_t T, uint32_t R, uint32_t per, uint32_t slots,
+                                             uint32_t slot_cap, uint32_t slots1, uint32_t slot_cap1,
+                                             PackSmem& S, uint8_t* out, uint64_t P, uint32_t raw,
+                                             uint32_t* const* bmap) {
   constexpr int G = PTraits<DT>::G, V = PTraits<DT>::V, ES = 16 / V;
   const uint32_t nfull = nb / 16u, t = gmod(nfull, T), k = gdiv(gdiv(nfull, T), per);
+  __syncwarp();  // (another lane of the warp may have stored the bitmap word)
   if (threadIdx.x != gmod(k * T + t, blockDim.x)) return;
   const uint32_t valid = (nb % 16u) / ES, ui = t * R + k;
-  const uint32_t slot = smem_u32(slots) + 4u * ui * slot_cap;
   uint32_t g4[4][4];
   split_vec(DT, load_vec(src, base, nfull, nb), g4);
-  SlotWriter sw;  // continued from the unit's bits
-  sw.slot = slot;
-  sw.bits = S.sbits[ui];
-  sw.nacc = sw.bits & 31u;
-  sw.wi = sw.bits >> 5;
-  sw.cap = slot_cap;
-  sw.acc = sw.nacc && sw.wi < slot_cap ? lds32v(slot + 4u * sw.wi) >> (32u - sw.nacc) : 0u;
 #pragma unroll
-  for (int q = 0; q < V; q++)
-    if (q < (int)valid) {
-      const uint32_t cl = code_of(smem_u32(S.codes[0]), g4[0][q >> 2], q & 3);
-      sw.put(cl & 0xFFFFu, cl >> 16);
+  for (int g = 0; g < G; g++) {
+    if (g == 0 || (G == 2 && slot_cap1)) {
+      if (bmap[g]) {
+        uint32_t any = 0;
+#pragma unroll
+        for (int q = 0; q < V / 4; q++) any |= g4[g][q];
+        if (!any) continue;
+        atomicOr(&bmap[g][nfull >> 5], 1u << (nfull & 31));
+      }
+      SlotWriter sw;  // continued from the unit's bits
+      sw.cap = g ? slot_cap1 : slot_cap;
+      sw.slot = (g ? slots1 : slots) + 4u * ui * sw.cap;
+      sw.bits = S.part[g][ui];
+      sw.nacc = sw.bits & 31u;
+      sw.wi = sw.bits >> 5;
+      sw.acc = sw.nacc && sw.wi < sw.cap ? lds32v(sw.slot + 4u * sw.wi) >> (32u - sw.nacc) : 0u;
+#pragma unroll
+      for (int q = 0; q < V; q++)
+        if (q < (int)valid) {
+          const uint32_t cl = code_of(smem_u32(S.codes[g]), g4[g][q >> 2], q & 3);
+          sw.put(cl & 0xFFFFu, cl >> 16);
+        }
+      sw.finish();
+      if (g == 0) S.sbits[ui] = sw.bits;
+      S.part[g][ui] = sw.bits;
+    } else if (raw >> g & 1u) {
+      uint8_t* p = out + P + S.off[g];
+      if (V == 8) reinterpret_cast<uint2*>(p)[nfull] = make_uint2(g4[g][0], g4[g][1]);
+      else reinterpret_cast<uint32_t*>(p)[nfull] = g4[g][0];
     }
-  sw.finish();
-  S.sbits[ui] = sw.bits;
-  S.part[0][ui] = sw.bits;
-#pragma unroll
-  for (int g = 1; g < G; g++) {
-    if (!(raw >> g & 1u)) continue;
-    uint8_t* p = out + P + S.off[g];
-    if (V == 8) reinterpret_cast<uint2*>(p)[nfull] = make_uint2(g4[g][0], g4[g][1]);
-    else reinterpret_cast<uint32_t*>(p)[nfull] = g4[g][0];
   }
 }
 
@@ -1612,6 +1745,43 @@ __device__ __forceinline__ void pass_b_whole(const PackSmem& S, const uint32_t* 
   for (uint32_t w = ((tot + 31) >> 5) + tid; w < capw; w += nthr) words[w] = 0;
 }
 
+// The same for units of any size that fits their slots of cap words at sl0 (a
+// word may span several units), offsets in part[0..units].
+#ifndef PBA
+#define PBA __forceinline__
+#endif
+__device__ PBA void pass_b_any(const uint32_t* part, uint32_t sl0, uint32_t cap,
+                                           uint32_t units, uint32_t* words, uint32_t capw) {
+  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, nwarps = nthr >> 5;
+  const uint32_t tot = part[units], used = min((tot + 31u) >> 5, capw);
+  const uint32_t upw = (units + (uint32_t)nwarps - 1) / (uint32_t)nwarps;
+  const uint32_t u0 = min(units, (uint32_t)(tid >> 5) * upw), u1 = min(units, u0 + upw);
+  if (u0 < u1) {
+    const uint32_t wend = u1 < units ? min((part[u1] + 31) >> 5, used) : used;
+    uint32_t cu = u0, o = part[u0], e = part[u0 + 1];
+    for (uint32_t w = ((o + 31) >> 5) + (uint32_t)lane; w < wend; w += 32) {
+      const uint32_t bit = 32u * w;
+      while (bit >= e) {
+        cu++;
+        o = e;
+        e = part[cu + 1];
+      }
+      const uint32_t k = bit - o, i = k >> 5, sl = sl0 + 4u * cu * cap;
+      const uint32_t a = lds32v(sl + 4u * i);
+      const uint32_t b = 32u * (i + 1) < e - o ? lds32v(sl + 4u * (i + 1)) : 0u;
+      uint32_t x = __funnelshift_l(b, a, k & 31), r = e - bit, ee = e;
+      for (uint32_t nu = cu + 1; r < 32 && nu < units; nu++) {
+        const uint32_t e2 = part[nu + 1];
+        if (e2 > ee) x |= lds32v(sl0 + 4u * nu * cap) >> r;
+        r += e2 - ee;
+        ee = e2;
+      }
+      words[w] = x;
+    }
+  }
+  for (uint32_t w = used + tid; w < capw; w += nthr) words[w] = 0;
+}
+
 template <int DT, bool S2>
 __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t* slots,
                                 const uint8_t* const* tabp) {
@@ -1693,9 +1863,15 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
   if (!(slot_cap & 1u)) slot_cap--;
   const uint32_t slots1 = smem_u32(slots) + 4u * units * slot_cap;  // second group's slots
   const bool fast_a = sg == 0 && huff == 1u && sparse == 0;
+  // both 16-bit groups coded and staged (deltas)
+  bool coded_a = S2 && G == 2 && sg == 0 && sg1 == 1 && base && T % 32 == 0;
   bool pairs = false;
   if constexpr (DT == ZIPNN_BF16 || DT == ZIPNN_FP16 || DT == ZIPNN_FP32)
-    pairs = fast_a && smem_u32(S.ptab) + 4096u <= 65536u && build_pair_table(S);
+    pairs = (fast_a || coded_a) && smem_u32(S.ptab) + 4096u <= 65536u && build_pair_table(S);
+  coded_a = coded_a && pairs;
+  if (coded_a)
+    for (int i = tid; i < 256; i += nthr)
+      S.etab[i] = ((S.codes[1][i] & 0xFFFFu) << 6) | (S.codes[1][i] >> 16);
   __syncthreads();
 
   // pass A: unit bits (+ raw planes, + slot encoding of group sg)
@@ -1706,10 +1882,25 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
     }
     if (!pairs)
       pack_fast_a<DT>(src, base, (uint32_t)nb / 16u, T, R, (uint32_t)per, slots, slot_cap, S, out, P, raw);
-    if (nb % 16)
-      pack_partial<DT>(src, base, (uint32_t)nb, T, R, (uint32_t)per, slots, slot_cap, S, out, P, raw);
+  } else if (coded_a) {
+    if constexpr (S2 && G == 2) {
+      const uint4* s4 = reinterpret_cast<const uint4*>(src);
+      const uint4* b4 = reinterpret_cast<const uint4*>(base);
+      const uint32_t nf = (uint32_t)nb / 16u, sl = smem_u32(slots), pv = (uint32_t)per;
+      if (sparse == 3u)
+        pack_coded_a<true, true>(s4, b4, nf, T, R, pv, sl, slot_cap, slots1, slot_cap1, S, bmap[0], bmap[1]);
+      else if (sparse == 1u)
+        pack_coded_a<true, false>(s4, b4, nf, T, R, pv, sl, slot_cap, slots1, slot_cap1, S, bmap[0], bmap[1]);
+      else if (sparse == 2u)
+        pack_coded_a<false, true>(s4, b4, nf, T, R, pv, sl, slot_cap, slots1, slot_cap1, S, bmap[0], bmap[1]);
+      else
+        pack_coded_a<false, false>(s4, b4, nf, T, R, pv, sl, slot_cap, slots1, slot_cap1, S, bmap[0], bmap[1]);
+    }
   }
-  for (uint32_t u = fast_a ? units : tid; u < units; u += nthr) {
+  if ((fast_a || coded_a) && nb % 16)
+    pack_partial<DT>(src, base, (uint32_t)nb, T, R, (uint32_t)per, smem_u32(slots), slot_cap, slots1,
+                     coded_a ? slot_cap1 : 0u, S, out, P, raw, bmap);
+  for (uint32_t u = fast_a || coded_a ? units : tid; u < units; u += nthr) {
     const uint32_t t = gmod(u, T), k = gdiv(u, T);
     uint32_t bits[G];
 #pragma unroll
@@ -1827,9 +2018,10 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
     for (uint64_t q = m + tid; q < align_up(m, 16); q += nthr) p[q] = 0;
   }
   if (!huff) return;
-  // Pass B writes each output word of the slot-staged group whole (no zeroed
-  // words, no atomics) when that group is the only coded one and every unit
-  // holds 32 to slot_cap * 32 bits (so a word spans at most two units)
+  // Pass B writes each output word of the staged groups whole (no zeroed words,
+  // no atomics) when every coded group is staged and every unit fits its slot:
+  // pass_b_whole when there is one group, a unit per thread and 32 bits or more
+  // in each (so a word spans at most two units), else pass_b_any
   bool whole = sg == 0 && huff == 1u;
   // one unit per thread (unit tid): its exclusive bit offset from a warp scan
   // before this barrier and a scan of the warp totals after it
@@ -1846,14 +2038,9 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
       if (lane >= o) uincl += t;
     }
     if (lane == 31) S.wsum[wid] = uincl;
-  } else {
-    for (uint32_t u = tid; whole && u < units; u += nthr) {
-      const uint32_t b = S.sbits[gmod(u, T) * R + gdiv(u, T)];
-      whole = b >= 32u && b <= slot_cap * 32u;
-    }
   }
-  whole = __syncthreads_and(whole) != 0;
-  if (whole && one) {
+  whole = __syncthreads_and(whole && one) != 0;
+  if (whole) {
     const int nw = nthr >> 5;
     const uint32_t ws = lane < nw ? S.wsum[lane] : 0u;
     uint32_t wi = ws;
@@ -1876,6 +2063,11 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
     return;
   }
 
+  bool fit = huff == ((sg >= 0 ? 1u << sg : 0u) | (sg1 >= 0 ? 1u << sg1 : 0u));
+  for (uint32_t u = tid; fit && u < units; u += nthr)
+    fit = S.sbits[u] <= slot_cap * 32u && (sg1 < 0 || S.part[sg1 < 0 ? 0 : sg1][u] <= slot_cap1 * 32u);
+  fit = __syncthreads_and(fit) != 0;
+
   // scan unit bits -> unit offsets; table bytes, sub-stream starts, zeroed words
 #pragma unroll
   for (int g = 0; g < G; g++) {
@@ -1890,7 +2082,7 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
     uint32_t* words = po + (T - 1);
     const uint32_t capw =
         (uint32_t)(align_up(S.meta[g].size, 16) - h - 4ull * nbm - 4ull * (T - 1)) / 4;
-    if (!whole)
+    if (!fit)
       for (uint32_t w = tid; w < capw; w += nthr) words[w] = 0;
     if (tid == 0) {
       S.capw[g] = capw;
@@ -1899,10 +2091,12 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
   }
   __syncthreads();
 
-  if (whole) {
-    pass_b_whole(S, slots, slot_cap, units,
-                 reinterpret_cast<uint32_t*>(out + P + S.off[0] + S.hsz[0]), S.capw[0],
-                 S.part[0][units - 1] + S.sbits[units - 1]);
+  if (fit) {
+#pragma unroll
+    for (int g = 0; g < G; g++)
+      if (g == sg || (S2 && g == sg1))
+        pass_b_any(S.part[g], g == sg ? smem_u32(slots) : slots1, g == sg ? slot_cap : slot_cap1, units,
+                   reinterpret_cast<uint32_t*>(out + P + S.off[g] + S.hsz[g]), S.capw[g]);
     return;
   }
 

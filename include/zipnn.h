@@ -225,6 +225,13 @@ zipnn_status zipnn_batch_compress_into_ex(
  * 64 bytes).  The stream does not own d_data.  ECORRUPT if the header is bad. */
 zipnn_status zipnn_stream_wrap(const void* d_data, size_t nbytes, zipnn_stream* out);
 
+/* zipnn_stream_wrap for a container that work queued on cuda_stream writes into a
+ * buffer of `capacity` bytes: copies the header on that stream, waits for the
+ * stream and takes the container's size from the header.  ECORRUPT if the
+ * header is bad or names more bytes than the buffer has. */
+zipnn_status zipnn_stream_read(const void* d_data, size_t capacity, zipnn_stream* out,
+                               void* cuda_stream);
+
 /* Original size and dtype of a container: the exact byte count that
  * decompression gives back (Sec. 2.3, "Lossless compression": compression
  * followed by decompression returns the input exactly), read from the header

@@ -445,6 +445,25 @@ zipnn_status zipnn_stream_wrap(const void* d_data, size_t nbytes, zipnn_stream* 
   return ZIPNN_OK;
 }
 
+zipnn_status zipnn_stream_read(const void* d_data, size_t capacity, zipnn_stream* out,
+                               void* cuda_stream) {
+  if (!out || !d_data || !aligned16(d_data) || capacity < (size_t)kHdrBytes) return ZIPNN_EINVAL;
+  memset(out, 0, sizeof(*out));
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  uint8_t h[kHdrBytes];
+  cudaError_t e = cudaMemcpyAsync(h, d_data, kHdrBytes, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return cuda_status(e);
+  uint64_t total;
+  memcpy(&total, h + 40, 8);
+  if (total > capacity) return ZIPNN_ECORRUPT;
+  zipnn_status rc = read_header(h, total, out);
+  if (rc) return rc;
+  out->data = const_cast<void*>(d_data);
+  out->owned = 0;
+  return ZIPNN_OK;
+}
+
 zipnn_status zipnn_decompressed_size(const zipnn_stream* s, size_t* nbytes, int* dtype) {
   if (!s) return ZIPNN_EINVAL;
   if (nbytes) *nbytes = s->orig_nbytes;

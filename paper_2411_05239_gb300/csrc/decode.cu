@@ -108,9 +108,7 @@ cudaError_t launch_decode_ex(const Job* d_jobs, const Job* h_one, int njobs,
   if (h_one) r.one = *h_one;
   else memset(&r.one, 0, sizeof(Job));
   r.n = njobs;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const int want_threads = (tuning && tuning->threads) ? tuning->threads : 256;
   const int want_parts = tuning ? tuning->parts : 0;
   // Launches with few chunks split every chunk's sub-streams over `parts` work
@@ -133,16 +131,11 @@ cudaError_t launch_decode_ex(const Job* d_jobs, const Job* h_one, int njobs,
   const void* kern = shape.family == ZIPNN_BF16   ? decode_kernel_16(cfg.kind, threads, three)
                      : shape.family == ZIPNN_FP32 ? decode_kernel_32(cfg.kind, threads, three)
                                                   : decode_kernel_u8(cfg.kind, threads, three);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  // all of the unified L1 / shared array as shared memory, so the CTAs per
-  // SM that the occupancy query reports are the ones that become resident
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                           cudaSharedmemCarveoutMaxShared);
-  if (e != cudaSuccess) return e;
+  // (all of the unified L1 / shared array as shared memory, so the CTAs per SM
+  // that the occupancy query reports are the ones that become resident)
   int occ = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
-  if (occ < 1) occ = 1;
+  const cudaError_t e = prepare_kernel(kern, smem, threads, &occ);
+  if (e != cudaSuccess) return e;
   int per_sm = tuning && tuning->ctas_per_sm > 0 ? tuning->ctas_per_sm : occ;
   if (per_sm > occ) per_sm = occ;
   uint64_t grid = (uint64_t)sms * per_sm;

@@ -1747,10 +1747,7 @@ __device__ __forceinline__ void pass_b_whole(const PackSmem& S, const uint32_t* 
 
 // The same for units of any size that fits their slots of cap words at sl0 (a
 // word may span several units), offsets in part[0..units].
-#ifndef PBA
-#define PBA __forceinline__
-#endif
-__device__ PBA void pass_b_any(const uint32_t* part, uint32_t sl0, uint32_t cap,
+__device__ __forceinline__ void pass_b_any(const uint32_t* part, uint32_t sl0, uint32_t cap,
                                            uint32_t units, uint32_t* words, uint32_t capw) {
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, nwarps = nthr >> 5;
   const uint32_t tot = part[units], used = min((tot + 31u) >> 5, capw);
@@ -2506,10 +2503,7 @@ cudaError_t launch_encode_analyse_ex(const Job* d_jobs, const Job* h_one, int nj
     const int hs = hist_smem_bytes(max_groups < 1 ? 4 : (max_groups > 4 ? 4 : max_groups));
     auto kh = pick(uniform_dtype, k_hist<ZIPNN_BF16>, k_hist<ZIPNN_FP16>, k_hist<ZIPNN_FP32>,
                    k_hist<ZIPNN_U8>, k_hist<-1>);
-    cudaError_t ea = cudaFuncSetAttribute(kh, cudaFuncAttributeMaxDynamicSharedMemorySize, hs);
-    if (ea == cudaSuccess)
-      ea = cudaFuncSetAttribute(kh, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                cudaSharedmemCarveoutMaxShared);
+    const cudaError_t ea = prepare_kernel(reinterpret_cast<const void*>(kh), hs);
     if (ea != cudaSuccess) return ea;
     kh<<<(unsigned)nchunks_total, kHistThreads, hs, st>>>(r, s.hist, s.zsyms);
     unsigned nb = (unsigned)((ngc_total + kBuildWarps - 1) / kBuildWarps);
@@ -2536,10 +2530,7 @@ cudaError_t launch_encode_pack_ex(const Job* d_jobs, const Job* h_one, int njobs
                              k_pack<ZIPNN_FP32, false>, k_pack<ZIPNN_U8, false>,
                              k_pack<-1, false>);
   const int ps = (int)(kPackSlotWords * 4);
-  cudaError_t ea = cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, ps);
-  if (ea == cudaSuccess)
-    ea = cudaFuncSetAttribute(kp, cudaFuncAttributePreferredSharedMemoryCarveout,
-                              cudaSharedmemCarveoutMaxShared);
+  const cudaError_t ea = prepare_kernel(reinterpret_cast<const void*>(kp), ps);
   if (ea != cudaSuccess) return ea;
   kp<<<(unsigned)(nchunks_total + njobs), kPackThreads, ps, st>>>(r, nchunks_total, s.codes, s.tabs,
                                                                 s.meta, s.offs, s.totals);
@@ -2567,16 +2558,10 @@ cudaError_t launch_encode_fused(const Job* d_jobs, const Job* h_one, int njobs,
                      : dtype == ZIPNN_FP16 ? reinterpret_cast<const void*>(k_compress<ZIPNN_FP16>)
                                            : reinterpret_cast<const void*>(k_compress<ZIPNN_U8>);
   const int dynb = (int)kFusedDynBytes;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dynb);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
+  int occ = 0;
+  e = prepare_kernel(kern, dynb, kPackThreads, &occ);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, occ = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kPackThreads, dynb);
-  if (occ < 1) occ = 1;
+  const int sms = device_sms();
   const uint64_t items = nchunks_total + (uint64_t)njobs;
   uint64_t grid = (uint64_t)sms * (uint64_t)occ;
   if (grid > items) grid = items;

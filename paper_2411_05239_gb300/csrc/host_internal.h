@@ -57,6 +57,15 @@ cudaError_t launch_encode(const Job* d_jobs, const Job* h_one, int njobs, uint64
                           bool any_delta = false);
 bool fused_encoder_applies(int dtype, bool any_skip);
 
+// Launch settings that only a kernel and its shared memory decide, asked of
+// the runtime once per device and kept (launch_setup.cu): room for smem bytes of
+// dynamic shared memory, all of the unified L1 / shared array as shared
+// memory, and, where wanted, the CTAs per SM (at least 1).
+cudaError_t prepare_kernel(const void* kern, int smem, int threads = 0,
+                           int* ctas_per_sm = nullptr);
+// SMs of the current device.
+int device_sms();
+
 // Decoder (decode.cu): one persistent launch per dtype family over all chunks
 // of its jobs.  What a launch needs to know of its jobs, gathered with add():
 struct DecodeShape {

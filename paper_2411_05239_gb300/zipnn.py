@@ -33,7 +33,7 @@ EXPORTS = [
     "zipnn_batch_compress_workspace_size", "zipnn_batch_compress_into",
     "zipnn_plan_decompress", "zipnn_plan_compress", "zipnn_plan_launch", "zipnn_plan_destroy",
     "zipnn_plan_load", "zipnn_batch_compress_into_ex", "zipnn_partition_chunks",
-    "zipnn_plan_decompress_range",
+    "zipnn_plan_decompress_range", "zipnn_stream_read",
 ]
 
 
@@ -87,6 +87,7 @@ def lib() -> ctypes.CDLL:
         "zipnn_delta": ([vp, vp, sz, i32, sz, zsp, vp], i32),
         "zipnn_compress_into": ([vp, vp, sz, i32, sz, u32, vp, sz, vp, sz, vp, vp], i32),
         "zipnn_stream_wrap": ([vp, sz, zsp], i32),
+        "zipnn_stream_read": ([vp, sz, zsp, vp], i32),
         "zipnn_decompressed_size": ([zsp, ctypes.POINTER(sz), ctypes.POINTER(i32)], i32),
         "zipnn_decompress": ([zsp, vp, vp, sz, vp], i32),
         "zipnn_batch_decompress": ([zsp, ctypes.POINTER(vp), ctypes.POINTER(vp), i32,
@@ -132,8 +133,10 @@ def _check(rc: int, what: str) -> None:
 
 
 def _sp(stream) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    # the current stream's handle without building a Stream object
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 class _CudaView:
@@ -205,6 +208,16 @@ def _flat_u8(x: torch.Tensor) -> torch.Tensor:
     return x.contiguous().view(-1).view(torch.uint8)
 
 
+def _span(x: torch.Tensor) -> tuple[int, int, torch.Tensor]:
+    """(pointer, bytes, tensor that owns them) of x's elements in order.  The
+    byte views of _flat_u8 cost as much host time as the launch of a small
+    decode; contiguous tensors of the codec's own types need none of them."""
+    if x.is_cuda and x.dtype in TORCH_TO_CODE and x.is_contiguous() and not x.is_neg():
+        return x.data_ptr(), x.numel() * x.element_size(), x
+    u = _flat_u8(x)
+    return u.data_ptr(), u.numel(), u
+
+
 def dtype_code(x: torch.Tensor, dtype: int | None) -> int:
     if dtype is not None:
         return dtype
@@ -231,14 +244,14 @@ def compress_into(x: torch.Tensor, out: torch.Tensor, workspace: torch.Tensor,
                   stream=None) -> None:
     """Enqueue compression of x into the caller's buffers (no allocation, no sync)."""
     code = dtype_code(x, dtype)
-    src = _flat_u8(x)
-    bp = _flat_u8(base).data_ptr() if base is not None else None
-    if base is not None and base.numel() * base.element_size() != src.numel():
+    sp, n, src = _span(x)
+    bp, nb, b = _span(base) if base is not None else (None, n, None)
+    if nb != n:
         raise ValueError("base size differs")
     onp = out_nbytes.data_ptr() if out_nbytes is not None else None
-    rc = lib().zipnn_compress_into(src.data_ptr() if src.numel() else None, bp, src.numel(), code,
-                                   chunk_bytes, lanes, out.data_ptr(), out.numel(),
-                                   workspace.data_ptr(), workspace.numel(), onp, _sp(stream))
+    rc = lib().zipnn_compress_into(sp if n else None, bp, n, code, chunk_bytes, lanes,
+                                   out.data_ptr(), out.numel(), workspace.data_ptr(),
+                                   workspace.numel(), onp, _sp(stream))
     _check(rc, "zipnn_compress_into")
 
 
@@ -246,17 +259,23 @@ def compress(x: torch.Tensor, chunk_bytes: int = DEFAULT_CHUNK, lanes: int = 0,
              base: torch.Tensor | None = None, dtype: int | None = None, stream=None,
              exact: bool = True) -> Compressed:
     """Compress a CUDA tensor; the container lives in a torch-allocated buffer.
-    Reads the container size back (one synchronisation)."""
+    Reads the container's header back, whose size the exact copy needs, and
+    returns when the container is complete."""
     code = dtype_code(x, dtype)
     n = x.numel() * x.element_size()
     out = torch.empty(compress_bound(n, code, chunk_bytes), dtype=torch.uint8, device=x.device)
     ws = torch.empty(workspace_size(n, code, chunk_bytes), dtype=torch.uint8, device=x.device)
-    onb = torch.zeros(1, dtype=torch.int64, device=x.device)
-    compress_into(x, out, ws, onb, base=base, chunk_bytes=chunk_bytes, lanes=lanes, dtype=code,
+    compress_into(x, out, ws, None, base=base, chunk_bytes=chunk_bytes, lanes=lanes, dtype=code,
                   stream=stream)
-    total = int(onb.item())
-    buf = out[:total].clone() if exact else out
-    return wrap(buf, total)
+    zs = ZStream()
+    _check(lib().zipnn_stream_read(out.data_ptr(), out.numel(), ctypes.byref(zs), _sp(stream)),
+           "zipnn_stream_read")
+    if not exact:
+        return Compressed(zs, out)
+    buf = out[:zs.nbytes].clone()
+    zs.data = buf.data_ptr()
+    torch.cuda.current_stream().synchronize()
+    return Compressed(zs, buf)
 
 
 def compress_lib(x: torch.Tensor, chunk_bytes: int = DEFAULT_CHUNK, base: torch.Tensor | None = None,
@@ -300,10 +319,9 @@ def decompress(c: Compressed, out: torch.Tensor | None = None, base: torch.Tenso
     if out is None:
         out = torch.empty(c.orig_nbytes // ELEM_SIZE[c.dtype_code],
                           dtype=CODE_TO_TORCH[c.dtype_code], device="cuda")
-    o = _flat_u8(out)
-    bp = _flat_u8(base).data_ptr() if base is not None else None
-    rc = lib().zipnn_decompress(ctypes.byref(c.zs), bp, o.data_ptr() if o.numel() else None,
-                                o.numel(), _sp(stream))
+    op, n, o = _span(out)
+    bp, _, b = _span(base) if base is not None else (None, 0, None)
+    rc = lib().zipnn_decompress(ctypes.byref(c.zs), bp, op if n else None, n, _sp(stream))
     _check(rc, "zipnn_decompress")
     return out
 
@@ -319,11 +337,8 @@ def batch_decompress(cs: list[Compressed], outs: list[torch.Tensor],
     """Decode many containers in one persistent launch (device work queue)."""
     n = len(cs)
     arr = (ZStream * n)(*[c.zs for c in cs])
-    dsts = (ctypes.c_void_p * n)(*[_flat_u8(o).data_ptr() for o in outs])
-    bp = None
-    if bases is not None:
-        bp = (ctypes.c_void_p * n)(*[(_flat_u8(b).data_ptr() if b is not None else None)
-                                     for b in bases])
+    dsts = _ptrs(outs)
+    bp = _ptrs(bases) if bases is not None else None
     rc = lib().zipnn_batch_decompress(arr, bp, dsts, n, ctypes.byref(tune) if tune else None,
                                       _sp(stream))
     _check(rc, "zipnn_batch_decompress")
@@ -336,8 +351,7 @@ def sync_status(stream=None) -> None:
 
 def _ptrs(ts, allow_none=False):
     n = len(ts)
-    return (ctypes.c_void_p * n)(*[(_flat_u8(t).data_ptr() if t is not None else None)
-                                   for t in ts])
+    return (ctypes.c_void_p * n)(*[(_span(t)[0] if t is not None else None) for t in ts])
 
 
 class BatchCompressor:

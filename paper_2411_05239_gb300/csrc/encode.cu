@@ -407,31 +407,11 @@ static int hist_smem_bytes(int max_groups) {
 // k_build: one warp per group-chunk.
 
 struct BuildSmem {
-  uint32_t leafw[256];    // leaf weights, sorted by (count asc, symbol desc)
-  uint8_t leafsym[256];
-  uint8_t lens[256];      // code length per symbol
-  uint32_t lst[2][512];   // package-merge lists (double buffer)
-  uint32_t pk[256];       // packages of the previous list
-  uint32_t leafbits[kMaxLen][16];  // which positions of list i are leaves
+  uint8_t lens[256];            // code length per symbol
   uint32_t keys[256];
+  uint32_t lst[2][64];          // package-merge lists of up to 32 symbols (double buffer)
+  uint32_t mask[kMaxLen][32];   // of more symbols: which of a lane's list items are leaves
 };
-
-__device__ __forceinline__ int upper_bound_u32(const uint32_t* a, int n, uint32_t x) {
-  int lo = 0, hi = n;  // first index with a[i] > x
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (a[mid] <= x) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-__device__ __forceinline__ int lower_bound_u32(const uint32_t* a, int n, uint32_t x) {
-  int lo = 0, hi = n;  // first index with a[i] >= x
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (a[mid] < x) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
 
 // Shannon bound: any prefix code spends >= sum c log2(n / c) bits on counts c
 // summing to n.  A lower bound of the size of such a code's payload with
@@ -505,12 +485,148 @@ __device__ void pm_lengths_small(BuildSmem& S, uint32_t key, uint32_t nz, int la
   __syncwarp();
 }
 
+constexpr uint32_t kPad = 0xFFFFFFFFu;  // larger than any key and any weight
+
+// Ascending order over lanes: v[r] of lane l is element R l + r.  With N = 32 R
+// elements of a bitonic sequence these are the steps from distance `from` down.
+template <int R>
+__device__ __forceinline__ void bitonic_clean(uint32_t v[R], int lane, int from) {
+#pragma unroll
+  for (int d = 16 * R; d >= R; d >>= 1) {
+    if (d > from) continue;
+    const int ls = d / R;  // partner lane distance
+    const bool upper = lane & ls;
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const uint32_t o = __shfl_xor_sync(0xffffffffu, v[r], ls);
+      v[r] = upper ? max(v[r], o) : min(v[r], o);
+    }
+  }
+#pragma unroll
+  for (int d = R / 2; d > 0; d >>= 1) {
+    if (d > from) continue;
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      if (r & d) continue;
+      const uint32_t a = v[r], b = v[r | d];
+      v[r] = min(a, b);
+      v[r | d] = max(a, b);
+    }
+  }
+}
+
+// Sorts the 32 R elements of a warp (same order as above): every merge first
+// compares each half with the mirror image of its partner, which leaves two
+// bitonic halves, whatever the sizes.
+template <int R>
+__device__ __forceinline__ void bitonic_sort(uint32_t v[R], int lane) {
+#pragma unroll
+  for (int size = 2; size <= 32 * R; size <<= 1) {
+    if (size <= R) {
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const int q = r ^ (size - 1);
+        if (q < r) continue;
+        const uint32_t a = v[r], b = v[q];
+        v[r] = min(a, b);
+        v[q] = max(a, b);
+      }
+    } else {
+      const int ls = size / R - 1;  // mirrored lane distance
+      const bool upper = lane & (size / R / 2);
+      uint32_t o[R];
+#pragma unroll
+      for (int r = 0; r < R; r++) o[r] = __shfl_xor_sync(0xffffffffu, v[R - 1 - r], ls);
+#pragma unroll
+      for (int r = 0; r < R; r++) v[r] = upper ? max(v[r], o[r]) : min(v[r], o[r]);
+    }
+    bitonic_clean<R>(v, lane, size / 4);
+  }
+}
+
+// Code lengths for 32 < nz <= 32 R non-zero symbols: S.keys[0..nz) holds their
+// keys.  The lists stay in registers: a list has up to 64 R items, the lower
+// 32 R of them in lo[] and the others in hi[], both in lane order, so that the
+// packages of a list are sums of two registers of one lane.  A package sorts
+// as 2 weight + 1 and a leaf as 2 weight (a leaf goes before a package of equal
+// weight), and the merge of the leaves with the packages is one bitonic
+// network: leaf i against package 32 R - 1 - i, then both halves.  88 shuffles
+// a level for 256 symbols and no dependent loads.  (Merging the lists in shared
+// memory, lane by lane, took 84 us for 1526 delta chunks and 43 us for 382
+// U8 chunks.)
+template <int R>
+__device__ __noinline__ void pm_lengths_wide(BuildSmem& S, uint32_t nz, int lane) {
+  const int n = (int)nz;
+  constexpr int N = 32 * R, H = R / 2;
+  uint32_t v[R], lo[R], hi[R];
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const int i = R * lane + r;
+    v[r] = i < n ? S.keys[i] : kPad;
+  }
+  bitonic_sort<R>(v, lane);
+  // leaf weights; the symbols stay in the keys' low bytes
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    lo[r] = v[r] == kPad ? kPad : v[r] >> 8 << 1;
+    hi[r] = kPad;
+  }
+#pragma unroll 1
+  for (int lvl = 1; lvl < kMaxLen; lvl++) {
+    // the packages of the list: 16 R from each half
+    uint32_t pl[H], ph[H];
+#pragma unroll
+    for (int r = 0; r < H; r++) {
+      pl[r] = lo[2 * r + 1] == kPad ? kPad : ((lo[2 * r] >> 1) + (lo[2 * r + 1] >> 1)) << 1 | 1u;
+      ph[r] = hi[2 * r + 1] == kPad ? kPad : ((hi[2 * r] >> 1) + (hi[2 * r + 1] >> 1)) << 1 | 1u;
+    }
+    // leaf i = R lane + r meets package N - 1 - i, of ph in the lower lanes
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const int src = (31 - 2 * lane - (r >= H ? 1 : 0)) & 31, q = H - 1 - r % H;
+      const uint32_t x = __shfl_sync(0xffffffffu, ph[q], src);
+      const uint32_t y = __shfl_sync(0xffffffffu, pl[q], src);
+      const uint32_t p = lane < 16 ? x : y, w = v[r] == kPad ? kPad : v[r] >> 8 << 1;
+      lo[r] = min(w, p);
+      hi[r] = max(w, p);
+    }
+    bitonic_clean<R>(lo, lane, N / 2);
+    bitonic_clean<R>(hi, lane, N / 2);
+    uint32_t leaves = 0;
+#pragma unroll
+    for (int r = 0; r < R; r++) leaves |= (~lo[r] & 1u) << r | (~hi[r] & 1u) << (R + r);
+    S.mask[lvl][lane] = leaves;
+  }
+  // selection, from the last list down: the first `take` items of a list hold
+  // some leaves, and packages that select twice as many items of the next
+  int take = 2 * (n - 1);
+  uint32_t len[R];
+#pragma unroll
+  for (int r = 0; r < R; r++) len[r] = 0;
+#pragma unroll 1
+  for (int lvl = kMaxLen - 1; lvl >= 0; lvl--) {
+    int leaves = take;  // list 0 holds leaves only
+    if (lvl) {
+      const uint32_t nl = (uint32_t)min(max(take - R * lane, 0), R);
+      const uint32_t nh = (uint32_t)min(max(take - N - R * lane, 0), R);
+      const uint32_t first = ((1u << nl) - 1u) | ((1u << nh) - 1u) << R;
+      leaves = (int)__reduce_add_sync(0xffffffffu, __popc(S.mask[lvl][lane] & first));
+    }
+#pragma unroll
+    for (int r = 0; r < R; r++) len[r] += R * lane + r < leaves;
+    take = 2 * (take - leaves);
+  }
+#pragma unroll
+  for (int r = 0; r < R; r++)
+    if (R * lane + r < n) S.lens[255u - (v[r] & 0xFFu)] = (uint8_t)len[r];
+  __syncwarp();
+}
+
 // Code lengths limited to kMaxLen bits for the counts cnt[k] of symbols
 // lane + 32 k (nz >= 2 of them non-zero), by package-merge; into S.lens.
 __device__ void pm_lengths(BuildSmem& S, const uint32_t cnt[8], uint32_t nz, int lane) {
-  // --- sort the leaves by key = count << 8 | (255 - symbol) (ascending):
-  // compact the non-zero symbols (ballot prefix), then rank each key among
-  // the nz compacted keys (keys are distinct: the symbol part differs)
+  // the leaves' keys count << 8 | (255 - symbol), which are distinct: the non-zero
+  // symbols one after another (ballot prefix)
   {
     uint32_t basek = 0;
     const uint32_t ltm = (1u << lane) - 1u;
@@ -524,156 +640,13 @@ __device__ void pm_lengths(BuildSmem& S, const uint32_t cnt[8], uint32_t nz, int
     }
   }
   __syncwarp();
-  if (nz <= 32) {
-    for (int k = 0; k < 8; k++)
-      if (!cnt[k]) S.lens[lane + 32 * k] = 0;
-    pm_lengths_small(S, lane < (int)nz ? S.keys[lane] : 0xFFFFFFFFu, nz, lane);
-    return;
-  }
-  if (nz <= 96) {
-    for (uint32_t i = lane; i < nz; i += 32) {
-      const uint32_t key = S.keys[i];
-      uint32_t r = 0;
-      for (uint32_t q = 0; q < nz; q++) r += (S.keys[q] < key);
-      S.leafw[r] = key >> 8;
-      S.leafsym[r] = (uint8_t)(255 - (key & 0xFFu));
-    }
-  } else {
-    // many leaves: a bitonic sort of the keys padded to 256 with the largest
-    // key (element i = 8 * lane + r in register r of the lane; partners 8 or
-    // more apart are exchanged by shuffles), instead of nz compares per key
-    uint32_t v[8];
-#pragma unroll
-    for (int r = 0; r < 8; r++) {
-      const uint32_t i = 8u * lane + r;
-      v[r] = i < nz ? S.keys[i] : 0xFFFFFFFFu;
-    }
-#pragma unroll
-    for (int size = 2; size <= 256; size <<= 1) {
-#pragma unroll
-      for (int stride = size >> 1; stride > 0; stride >>= 1) {
-        if (stride >= 8) {
-          const int ls = stride >> 3;  // partner lane distance
-#pragma unroll
-          for (int r = 0; r < 8; r++) {
-            const uint32_t i = 8u * lane + r;
-            const uint32_t o = __shfl_xor_sync(0xffffffffu, v[r], ls);
-            const bool up = (i & (uint32_t)size) == 0, lower = (lane & ls) == 0;
-            v[r] = (lower == up) ? min(v[r], o) : max(v[r], o);
-          }
-        } else {
-#pragma unroll
-          for (int r = 0; r < 8; r++) {
-            if (r & stride) continue;
-            const int q = r | stride;
-            const bool up = ((8u * lane + r) & (uint32_t)size) == 0;
-            const uint32_t a = v[r], b = v[q];
-            v[r] = up ? min(a, b) : max(a, b);
-            v[q] = up ? max(a, b) : min(a, b);
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < 8; r++) {
-      const uint32_t i = 8u * lane + r;
-      if (i < nz) {
-        S.leafw[i] = v[r] >> 8;
-        S.leafsym[i] = (uint8_t)(255 - (v[r] & 0xFFu));
-      }
-    }
-  }
-  for (int i = lane; i < kMaxLen * 16; i += 32) (&S.leafbits[0][0])[i] = 0;
-  __syncwarp();
-
-  // --- package-merge: list 0 = leaves; list i = merge(leaves, packages(list i-1))
-  const int n = (int)nz;
-  int sp = n;
-  uint32_t* prev = S.lst[0];
-  for (int k = lane; k < n; k += 32) prev[k] = S.leafw[k];
-  __syncwarp();
-  int cur_buf = 1;
-  for (int lvl = 1; lvl < kMaxLen; lvl++) {
-    uint32_t* cur = S.lst[cur_buf];
-    const int np = sp >> 1;
-    for (int k = lane; k < np; k += 32) S.pk[k] = prev[2 * k] + prev[2 * k + 1];
-    __syncwarp();
-    // the merged list, a leaf before a package of equal weight.  Few leaves:
-    // each package and leaf finds its position by a binary search in the
-    // other list.  Many (more than 96): merge path, lane l writes outputs
-    // [l * seg, (l + 1) * seg), one binary search finding how many leaves
-    // precede its first output, then a sequential merge that marks its
-    // leaves' positions (at most two bitmap words)
-    const int total = n + np, seg = (total + 31) >> 5;
-    const int d0 = min(total, lane * seg), d1 = min(total, d0 + seg);
-    if (n <= 96) {
-      for (int k = lane; k < np; k += 32) {
-        uint32_t w = S.pk[k];
-        cur[k + upper_bound_u32(S.leafw, n, w)] = w;      // after leaves of equal weight
-      }
-      for (int k = lane; k < n; k += 32) {
-        uint32_t w = S.leafw[k];
-        int pos = k + lower_bound_u32(S.pk, np, w);
-        cur[pos] = w;
-        atomicOr(&S.leafbits[lvl][pos >> 5], 1u << (pos & 31));
-      }
-    } else if (d0 < d1) {
-      int lo = max(0, d0 - np), hi = min(d0, n);
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (S.leafw[mid] <= S.pk[d0 - mid - 1]) lo = mid + 1; else hi = mid;
-      }
-      int li = lo, pi = d0 - lo;
-      uint64_t mask = 0;  // leaf positions from word d0 / 32
-      const int off = d0 & 31;
-      for (int d = d0; d < d1; d++) {
-        const bool leaf = pi >= np || (li < n && S.leafw[li] <= S.pk[pi]);
-        cur[d] = leaf ? S.leafw[li] : S.pk[pi];
-        if (leaf) {
-          mask |= 1ull << (off + d - d0);
-          li++;
-        } else {
-          pi++;
-        }
-      }
-      if ((uint32_t)mask) atomicOr(&S.leafbits[lvl][d0 >> 5], (uint32_t)mask);
-      if (mask >> 32) atomicOr(&S.leafbits[lvl][(d0 >> 5) + 1], (uint32_t)(mask >> 32));
-    }
-    __syncwarp();
-    sp = total;
-    prev = cur;
-    cur_buf ^= 1;
-  }
-
-  // --- selection, from the last list down: a[i] leaves and p packages among
-  // the first c items; the packages select the first 2p items of list i-1.
-  int a[kMaxLen];
-  {
-    int take = 2 * (n - 1);
-    for (int lvl = kMaxLen - 1; lvl >= 1; lvl--) {
-      int leaves = 0;
-      for (int wv = 0; wv < 16; wv++) {
-        int lo = wv * 32;
-        if (lo >= take) break;
-        uint32_t bits = S.leafbits[lvl][wv];
-        int upto = take - lo;
-        if (upto < 32) bits &= (1u << upto) - 1u;
-        leaves += __popc(bits);
-      }
-      a[lvl] = leaves;
-      take = 2 * (take - leaves);
-    }
-    a[0] = take;  // list 0 holds leaves only
-  }
-  for (int k = lane; k < n; k += 32) {
-    int len = 0;
-    for (int lvl = 0; lvl < kMaxLen; lvl++) len += (k < a[lvl]);
-    S.lens[S.leafsym[k]] = (uint8_t)len;
-  }
   for (int k = 0; k < 8; k++)
     if (!cnt[k]) S.lens[lane + 32 * k] = 0;
-  __syncwarp();
-
+  // the fewest registers a lane that hold the leaves
+  if (nz <= 32) pm_lengths_small(S, lane < (int)nz ? S.keys[lane] : kPad, nz, lane);
+  else if (nz <= 64) pm_lengths_wide<2>(S, nz, lane);
+  else if (nz <= 128) pm_lengths_wide<4>(S, nz, lane);
+  else pm_lengths_wide<8>(S, nz, lane);
 }
 
 // Mode decision, length-limited code and canonical table of one group-chunk

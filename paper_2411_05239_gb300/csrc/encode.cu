@@ -24,6 +24,9 @@ namespace zipnn {
 namespace {
 
 constexpr int kHistThreads = 256;
+// with up to one chunk per SM (an 8 MiB tensor: 32): the SM has no other CTA to
+// fill the time that one waits
+constexpr int kHistThreadsFew = 1024;
 constexpr int kBuildWarps = 4;
 
 struct JobRef {
@@ -283,7 +286,47 @@ __device__ void hist_chunk(const Job& J, uint64_t c, uint32_t* sh, uint32_t* his
       __syncthreads();
     }
     const uint64_t rend = min(nvec, r0 + rlen);
-    for (uint64_t v0 = r0 + (uint64_t)tid; v0 < rend; v0 += (uint64_t)NT * U) {
+    uint64_t rv = r0;
+    if constexpr (PK) {
+      // whole rounds of NT * U whole vectors: no bounds, prefetched like the
+      // 16-bit ones
+      const uint64_t nfast = r0 + (min(rend, nb / 16) - r0) / ((uint64_t)NT * U) * (NT * U);
+      for (uint64_t vp = r0 + tid + (uint64_t)NT * U; vp < nfast && vp < r0 + 2ull * NT * U; vp += NT) {
+        prefetch_l2(reinterpret_cast<const uint4*>(src) + vp);
+        if (base) prefetch_l2(reinterpret_cast<const uint4*>(base) + vp);
+      }
+      for (uint64_t v0 = r0 + tid; v0 < nfast; v0 += (uint64_t)NT * U) {
+        uint4 a[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          const uint64_t v = v0 + (uint64_t)u * NT;
+          const uint64_t vp = v + 2ull * NT * U;  // two rounds ahead
+          if (vp < nfast) {
+            prefetch_l2(reinterpret_cast<const uint4*>(src) + vp);
+            if (base) prefetch_l2(reinterpret_cast<const uint4*>(base) + vp);
+          }
+          a[u] = __ldg(reinterpret_cast<const uint4*>(src) + v);
+          if (base) {
+            const uint4 b = __ldg(reinterpret_cast<const uint4*>(base) + v);
+            a[u].x ^= b.x; a[u].y ^= b.y; a[u].z ^= b.z; a[u].w ^= b.w;
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          hist32_elem(hls, a[u].x);
+          hist32_elem(hls, a[u].y);
+          hist32_elem(hls, a[u].z);
+          hist32_elem(hls, a[u].w);
+          const uint32_t any = a[u].x | a[u].y | a[u].z | a[u].w;
+          if (!(any & 0x7F800000u)) zc[0] += 4;
+          if (!(any & 0x807F0000u)) zc[1 % G] += 4;
+          if (!(any & 0x0000FF00u)) zc[2 % G] += 4;
+          if (!(any & 0x000000FFu)) zc[3 % G] += 4;
+        }
+      }
+      rv = nfast;
+    }
+    for (uint64_t v0 = rv + (uint64_t)tid; v0 < rend; v0 += (uint64_t)NT * U) {
       uint4 a[U];
 #pragma unroll
       for (int u = 0; u < U; u++) {
@@ -295,20 +338,6 @@ __device__ void hist_chunk(const Job& J, uint64_t c, uint32_t* sh, uint32_t* his
         const uint64_t v = v0 + (uint64_t)u * NT;
         if (v >= rend) break;
         const int valid = (v + 1) * V <= m ? V : (int)(m - v * V);
-        if constexpr (PK) {
-          if (valid == V) {  // four whole elements
-            hist32_elem(hls, a[u].x);
-            hist32_elem(hls, a[u].y);
-            hist32_elem(hls, a[u].z);
-            hist32_elem(hls, a[u].w);
-            const uint32_t any = a[u].x | a[u].y | a[u].z | a[u].w;
-            if (!(any & 0x7F800000u)) zc[0] += 4;
-            if (!(any & 0x807F0000u)) zc[1 % G] += 4;
-            if (!(any & 0x0000FF00u)) zc[2 % G] += 4;
-            if (!(any & 0x000000FFu)) zc[3 % G] += 4;
-            continue;
-          }
-        }
         uint32_t g[4][4];
         split_vec(DT, a[u], g);
 #pragma unroll
@@ -373,8 +402,8 @@ __device__ void hist_chunk(const Job& J, uint64_t c, uint32_t* sh, uint32_t* his
   __syncthreads();
 }
 
-template <int DTS>
-__global__ void __launch_bounds__(kHistThreads)
+template <int DTS, int NT>
+__global__ void __launch_bounds__(NT)
 k_hist(JobRef jr, uint32_t* __restrict__ hist, uint32_t* __restrict__ zsyms) {
   extern __shared__ uint32_t hsm[];
   const uint64_t chunk = blockIdx.x;
@@ -385,14 +414,14 @@ k_hist(JobRef jr, uint32_t* __restrict__ hist, uint32_t* __restrict__ zsyms) {
   uint32_t* ho = hist + gc0 * 256;
   uint32_t* zo = zsyms + gc0;
   if (DTS >= 0) {
-    hist_chunk<(DTS < 0 ? 0 : DTS)>(J, c, hsm, ho, zo);
+    hist_chunk<(DTS < 0 ? 0 : DTS), NT>(J, c, hsm, ho, zo);
     return;
   }
   switch (J.dtype) {
-    case ZIPNN_BF16: hist_chunk<ZIPNN_BF16>(J, c, hsm, ho, zo); break;
-    case ZIPNN_FP16: hist_chunk<ZIPNN_FP16>(J, c, hsm, ho, zo); break;
-    case ZIPNN_FP32: hist_chunk<ZIPNN_FP32>(J, c, hsm, ho, zo); break;
-    default: hist_chunk<ZIPNN_U8>(J, c, hsm, ho, zo); break;
+    case ZIPNN_BF16: hist_chunk<ZIPNN_BF16, NT>(J, c, hsm, ho, zo); break;
+    case ZIPNN_FP16: hist_chunk<ZIPNN_FP16, NT>(J, c, hsm, ho, zo); break;
+    case ZIPNN_FP32: hist_chunk<ZIPNN_FP32, NT>(J, c, hsm, ho, zo); break;
+    default: hist_chunk<ZIPNN_U8, NT>(J, c, hsm, ho, zo); break;
   }
 }
 
@@ -2474,11 +2503,16 @@ cudaError_t launch_encode_analyse_ex(const Job* d_jobs, const Job* h_one, int nj
   }
   if (nchunks_total) {
     const int hs = hist_smem_bytes(max_groups < 1 ? 4 : (max_groups > 4 ? 4 : max_groups));
-    auto kh = pick(uniform_dtype, k_hist<ZIPNN_BF16>, k_hist<ZIPNN_FP16>, k_hist<ZIPNN_FP32>,
-                   k_hist<ZIPNN_U8>, k_hist<-1>);
+    // up to one chunk per SM: four times the threads on each
+    const bool few = nchunks_total <= (uint64_t)device_sms();
+    constexpr int N = kHistThreads, F = kHistThreadsFew;
+    auto kh = few ? pick(uniform_dtype, k_hist<ZIPNN_BF16, F>, k_hist<ZIPNN_FP16, F>,
+                         k_hist<ZIPNN_FP32, F>, k_hist<ZIPNN_U8, F>, k_hist<-1, F>)
+                  : pick(uniform_dtype, k_hist<ZIPNN_BF16, N>, k_hist<ZIPNN_FP16, N>,
+                         k_hist<ZIPNN_FP32, N>, k_hist<ZIPNN_U8, N>, k_hist<-1, N>);
     const cudaError_t ea = prepare_kernel(reinterpret_cast<const void*>(kh), hs);
     if (ea != cudaSuccess) return ea;
-    kh<<<(unsigned)nchunks_total, kHistThreads, hs, st>>>(r, s.hist, s.zsyms);
+    kh<<<(unsigned)nchunks_total, few ? F : N, hs, st>>>(r, s.hist, s.zsyms);
     unsigned nb = (unsigned)((ngc_total + kBuildWarps - 1) / kBuildWarps);
     k_build<<<nb, kBuildWarps * 32, 0, st>>>(r, ngc_total, s.hist, s.zsyms, s.codes, s.tabs,
                                              s.meta);

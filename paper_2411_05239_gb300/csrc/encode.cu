@@ -24,6 +24,8 @@ namespace zipnn {
 namespace {
 
 constexpr int kHistThreads = 256;
+// FP32 (112 KiB of counters, two CTAs per SM)
+constexpr int kHistThreadsWide = 512;
 // with up to one chunk per SM (an 8 MiB tensor: 32): the SM has no other CTA to
 // fill the time that one waits
 constexpr int kHistThreadsFew = 1024;
@@ -159,36 +161,36 @@ __device__ __forceinline__ void red_shared_add(uint32_t saddr, uint32_t v) {
   asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(saddr), "r"(v) : "memory");
 }
 
-// Histogram of one FP32 element x with packed counters: group g's counter of
-// bin b for this lane is the half b / 128 of the word at byte g * 16384 +
-// (b % 128) * 128 from hl (the shared-window address of lane 0's word of
-// group 0, bin 0, plus 4 * lane).  With g0 = x >> 23 & 0xFF, g1 = (x >> 24 &
-// 0x80) | (x >> 16 & 0x7F), g2 = x >> 8 & 0xFF and g3 = x & 0xFF, each word
-// offset is a shift and a mask of x and each half the bit 30, 31, 15 or 7
-// of x: no byte is extracted.
+// Histogram of one FP32 element x (hl: the shared-window address of lane 0's
+// counter of group 0, bin 0, plus 4 * lane).  With g0 = x >> 23 & 0xFF, g1 =
+// (x >> 24 & 0x80) | (x >> 16 & 0x7F) and g2 = x >> 8 & 0xFF, the counter
+// offsets are shifts and masks of x.  g3 = x & 0xFF has packed counters: bin
+// b is the half b / 128 of the word at (b % 128) * 128.
 __device__ __forceinline__ void hist32_elem(uint32_t hl, uint32_t x) {
-  red_shared_add(hl + ((x >> 16) & 0x3F80u), (x & 0x40000000u) ? 0x10000u : 1u);
-  red_shared_add(hl + 0x4000u + ((x >> 9) & 0x3F80u), (x & 0x80000000u) ? 0x10000u : 1u);
-  red_shared_add(hl + 0x8000u + ((x >> 1) & 0x3F80u), (x & 0x8000u) ? 0x10000u : 1u);
-  red_shared_add(hl + 0xC000u + ((x << 7) & 0x3F80u), (x & 0x80u) ? 0x10000u : 1u);
+  red_shared_inc(hl + ((x >> 16) & 0x7F80u));
+  red_shared_inc(hl + 0x8000u + (((x >> 17) & 0x4000u) | ((x >> 9) & 0x3F80u)));
+  red_shared_inc(hl + 0x10000u + ((x >> 1) & 0x7F80u));
+  red_shared_add(hl + 0x18000u + ((x << 7) & 0x3F80u), (x & 0x80u) ? 0x10000u : 1u);
 }
 
 // Histograms of chunk c of job J by the NT threads of the CTA, with the
 // lane-indexed counters in sh (hist_counter_words(DT) + G words); the bin
 // totals go to hist_out[g * 256 + b] and the symbols inside all-zero vectors
 // to zs_out[g] (global or shared memory).  Ends with every thread past a
-// barrier.  FP32 keeps two 16-bit counters per word (bins b and b + 128 of a
-// group and lane, low and high half): its four groups then take the 64 KiB
-// that two 16-bit groups take, three CTAs per SM instead of one.  A word
-// counts at most kPkRound / 8 symbols per half in a round of kPkRound vectors
-// (lane l of every warp adds into it: NT / 32 threads of kPkRound / NT
-// vectors each, 4 symbols per vector and group), so chunks of more than
+// barrier.  The last of FP32's four
+// groups keeps two 16-bit counters per word (bins b and b + 128 of a lane, low
+// and high half): the counters then take 112 KiB, two CTAs of 512 threads per
+// SM.  Adding a constant 1 is the faster shared-memory add, so only that group is
+// packed (all four, 64 KiB and three CTAs of 256 threads: 92 us for 256 MiB, now
+// 82).  A word counts at most kPkRound / 8 symbols per half in a round of
+// kPkRound vectors (lane l of every warp adds into it: NT / 32 threads of
+// kPkRound / NT vectors each, 4 symbols per vector), so chunks of more than
 // kPkRound vectors are counted in rounds, each round's halves added into
 // per-thread totals before the next.
 constexpr uint32_t kPkRound = 1u << 18;  // vectors (4 MiB) per round: <= 32768 per half
 template <int DT>
 __host__ __device__ constexpr int hist_counter_words() {
-  return DT == ZIPNN_FP32 ? 4 * 128 * 32 : (DT == ZIPNN_U8 ? 1 : 2) * 256 * 32;
+  return DT == ZIPNN_FP32 ? (3 * 256 + 128) * 32 : (DT == ZIPNN_U8 ? 1 : 2) * 256 * 32;
 }
 template <int DT, int NT = kHistThreads>
 __device__ void hist_chunk(const Job& J, uint64_t c, uint32_t* sh, uint32_t* hist_out,
@@ -252,22 +254,18 @@ __device__ void hist_chunk(const Job& J, uint64_t c, uint32_t* sh, uint32_t* his
     }
     vstart = nfast + tid;
   }
-  // packed counters: running totals of this thread's words (bins b, b + 128)
-  constexpr int PKW = PK ? (G * 128 + NT - 1) / NT : 1;
-  uint32_t tot_lo[PKW], tot_hi[PKW];
-#pragma unroll
-  for (int i = 0; i < PKW; i++) tot_lo[i] = tot_hi[i] = 0;
+  // packed counters: running totals of this thread's word (bins tid, tid + 128)
+  static_assert(!PK || NT >= 128, "a thread per packed word");
+  constexpr int FG = PK ? 3 : G;  // groups with whole counters
+  uint32_t* const packed = sh + FG * 256 * 32;
+  uint32_t tot_lo = 0, tot_hi = 0;
   auto add_packed = [&]() {
-#pragma unroll
-    for (int i = 0; i < PKW; i++) {
-      const int bw = tid + i * NT;
-      if (bw < G * 128) {
+    if (tid < 128) {
 #pragma unroll 8
-        for (int l = 0; l < 32; l++) {
-          const uint32_t w = sh[bw * 32 + ((l + bw) & 31)];
-          tot_lo[i] += w & 0xFFFFu;
-          tot_hi[i] += w >> 16;
-        }
+      for (int l = 0; l < 32; l++) {
+        const uint32_t w = packed[tid * 32 + ((l + tid) & 31)];
+        tot_lo += w & 0xFFFFu;
+        tot_hi += w >> 16;
       }
     }
   };
@@ -282,7 +280,7 @@ __device__ void hist_chunk(const Job& J, uint64_t c, uint32_t* sh, uint32_t* his
       __syncthreads();
       add_packed();
       __syncthreads();
-      for (int i = tid; i < CW; i += NT) sh[i] = 0;
+      for (int i = tid; i < 128 * 32; i += NT) packed[i] = 0;
       __syncthreads();
     }
     const uint64_t rend = min(nvec, r0 + rlen);
@@ -347,13 +345,11 @@ __device__ void hist_chunk(const Job& J, uint64_t c, uint32_t* sh, uint32_t* his
           for (int q = 0; q < V / 4; q++) any |= g[gg][q];
           if (!any) zc[gg] += (uint32_t)valid;   // bytes past the tail were loaded as zero
         }
-        // symbol b of group gg: word (gg * 256 + b) * 32 + lane, or with packed
-        // counters word (gg * 128 + b % 128) * 32 + lane, half b / 128
+        // symbol b of group gg: word (gg * 256 + b) * 32 + lane, or of packed
+        // counters word b % 128, half b / 128
         auto count = [&](int gg, uint32_t b) {
-          if constexpr (PK)
-            atomicAdd(&hl[(gg * 128 + (b & 127u)) * 32], (b & 128u) ? 0x10000u : 1u);
-          else
-            atomicAdd(&hl[(gg * 256 + b) * 32], 1u);
+          if (gg < FG) atomicAdd(&hl[(gg * 256 + b) * 32], 1u);
+          else atomicAdd(&packed[(b & 127u) * 32 + lane], (b & 128u) ? 0x10000u : 1u);
         };
         if (valid == V) {
 #pragma unroll
@@ -381,22 +377,17 @@ __device__ void hist_chunk(const Job& J, uint64_t c, uint32_t* sh, uint32_t* his
   if (tid < G) zs_out[tid] = zcnt[tid];
   // bin totals: thread b sums the 32 lane counters of bin b (rotated start so
   // the 32 threads of a warp read 32 different banks)
+  for (int b = tid; b < FG * 256; b += NT) {
+    uint32_t s = 0;
+#pragma unroll 8
+    for (int i = 0; i < 32; i++) s += sh[b * 32 + ((i + b) & 31)];
+    hist_out[b] = s;
+  }
   if constexpr (PK) {
     add_packed();
-#pragma unroll
-    for (int i = 0; i < PKW; i++) {
-      const int bw = tid + i * NT;
-      if (bw < G * 128) {
-        hist_out[(bw >> 7) * 256 + (bw & 127)] = tot_lo[i];
-        hist_out[(bw >> 7) * 256 + (bw & 127) + 128] = tot_hi[i];
-      }
-    }
-  } else {
-    for (int b = tid; b < G * 256; b += NT) {
-      uint32_t s = 0;
-#pragma unroll 8
-      for (int i = 0; i < 32; i++) s += sh[b * 32 + ((i + b) & 31)];
-      hist_out[b] = s;
+    if (tid < 128) {
+      hist_out[3 * 256 + tid] = tot_lo;
+      hist_out[3 * 256 + tid + 128] = tot_hi;
     }
   }
   __syncthreads();
@@ -425,11 +416,11 @@ k_hist(JobRef jr, uint32_t* __restrict__ hist, uint32_t* __restrict__ zsyms) {
   }
 }
 
-// counters + zero-symbol words: a launch that may hold FP32 chunks (packed
-// counters) needs as much as one of 16-bit chunks
+// counters + zero-symbol words
 static int hist_smem_bytes(int max_groups) {
-  const int g = max_groups > 2 ? 2 : max_groups;
-  return (g * 256 * 32 + max_groups) * 4;
+  const int words = max_groups > 2 ? hist_counter_words<ZIPNN_FP32>()
+                                   : max_groups * hist_counter_words<ZIPNN_U8>();
+  return (words + max_groups) * 4;
 }
 
 // ---------------------------------------------------------------------------
@@ -2503,16 +2494,19 @@ cudaError_t launch_encode_analyse_ex(const Job* d_jobs, const Job* h_one, int nj
   }
   if (nchunks_total) {
     const int hs = hist_smem_bytes(max_groups < 1 ? 4 : (max_groups > 4 ? 4 : max_groups));
-    // up to one chunk per SM: four times the threads on each
-    const bool few = nchunks_total <= (uint64_t)device_sms();
-    constexpr int N = kHistThreads, F = kHistThreadsFew;
+    // launches that may hold FP32 chunks have shared memory for two CTAs per SM
+    const bool few = nchunks_total <= (uint64_t)device_sms(), wide = max_groups > 2;
+    constexpr int N = kHistThreads, W = kHistThreadsWide, F = kHistThreadsFew;
     auto kh = few ? pick(uniform_dtype, k_hist<ZIPNN_BF16, F>, k_hist<ZIPNN_FP16, F>,
                          k_hist<ZIPNN_FP32, F>, k_hist<ZIPNN_U8, F>, k_hist<-1, F>)
-                  : pick(uniform_dtype, k_hist<ZIPNN_BF16, N>, k_hist<ZIPNN_FP16, N>,
-                         k_hist<ZIPNN_FP32, N>, k_hist<ZIPNN_U8, N>, k_hist<-1, N>);
+              : wide ? pick(uniform_dtype, k_hist<ZIPNN_BF16, N>, k_hist<ZIPNN_FP16, N>,
+                            k_hist<ZIPNN_FP32, W>, k_hist<ZIPNN_U8, N>, k_hist<-1, W>)
+                     : pick(uniform_dtype, k_hist<ZIPNN_BF16, N>, k_hist<ZIPNN_FP16, N>,
+                            k_hist<ZIPNN_FP32, W>, k_hist<ZIPNN_U8, N>, k_hist<-1, N>);
+    const int threads = few ? F : (wide && (uniform_dtype == ZIPNN_FP32 || uniform_dtype < 0)) ? W : N;
     const cudaError_t ea = prepare_kernel(reinterpret_cast<const void*>(kh), hs);
     if (ea != cudaSuccess) return ea;
-    kh<<<(unsigned)nchunks_total, few ? F : N, hs, st>>>(r, s.hist, s.zsyms);
+    kh<<<(unsigned)nchunks_total, threads, hs, st>>>(r, s.hist, s.zsyms);
     unsigned nb = (unsigned)((ngc_total + kBuildWarps - 1) / kBuildWarps);
     k_build<<<nb, kBuildWarps * 32, 0, st>>>(r, ngc_total, s.hist, s.zsyms, s.codes, s.tabs,
                                              s.meta);

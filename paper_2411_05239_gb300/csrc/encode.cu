@@ -15,6 +15,8 @@
 //               writes the map entries (and, in extra CTAs, the headers).
 #include <cstdint>
 #include <cstring>
+#include <initializer_list>
+
 #include <cuda_runtime.h>
 
 #include "host_internal.h"
@@ -122,6 +124,28 @@ __device__ __forceinline__ void split_vec(int dtype, uint4 a, uint32_t out[4][4]
     split16(a.x, a.y, out[0][0], out[1][0]);
     split16(a.z, a.w, out[0][1], out[1][1]);
   }
+}
+
+// ---------------------------------------------------------------------------
+// The encoder's kernels follow one another on a stream as programmatic
+// dependents: each lets the next one's CTAs start once its own are all
+// running (next_may_start), and each waits for the whole grid before it, memory
+// included, before it reads what that wrote.  A launch then costs its successor
+// little: a 48 KiB tensor takes 27.7 us like this and 31.2 with plain
+// launches, an 8 MiB one 37.4 and 45.7.
+
+__device__ __forceinline__ void next_may_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class T>
+__device__ __forceinline__ void opaque(T*& p) {
+  asm volatile("" : "+l"(p)::"memory");
+}
+// The pointers pass through the wait so that no load through them moves above it.
+template <class... P>
+__device__ __forceinline__ void wait_before(P&... p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  (void)std::initializer_list<int>{(opaque(p), 0)...};
 }
 
 // ---------------------------------------------------------------------------
@@ -397,6 +421,7 @@ template <int DTS, int NT>
 __global__ void __launch_bounds__(NT)
 k_hist(JobRef jr, uint32_t* __restrict__ hist, uint32_t* __restrict__ zsyms) {
   extern __shared__ uint32_t hsm[];
+  next_may_start();
   const uint64_t chunk = blockIdx.x;
   const int j = find_job_chunk(jr, chunk);
   const Job& J = job_at(jr, j);
@@ -814,10 +839,11 @@ __device__ void build_gc(const uint32_t* hist256, uint32_t zs, uint32_t m, uint3
 
 
 __global__ void __launch_bounds__(kBuildWarps * 32, 6)
-k_build(JobRef jr, uint64_t ngc_total, const uint32_t* __restrict__ hist,
-        const uint32_t* __restrict__ zsyms, uint32_t* __restrict__ codes,
-        uint8_t* __restrict__ tabs, GcMeta* __restrict__ meta) {
+k_build(JobRef jr, uint64_t ngc_total, const uint32_t* hist, const uint32_t* zsyms,
+        uint32_t* codes, uint8_t* tabs, GcMeta* meta) {
   __shared__ BuildSmem smem[kBuildWarps];
+  next_may_start();
+  wait_before(hist, zsyms);
   const int wid = threadIdx.x >> 5;
   const uint64_t gc = (uint64_t)blockIdx.x * kBuildWarps + wid;
   if (gc >= ngc_total) return;
@@ -841,9 +867,10 @@ k_build(JobRef jr, uint64_t ngc_total, const uint32_t* __restrict__ hist,
 constexpr int kScanThreads = 1024;
 
 __global__ void __launch_bounds__(kScanThreads)
-k_scan(JobRef jr, GcMeta* __restrict__ meta, uint64_t* __restrict__ offs,
-       uint64_t* __restrict__ totals, uint32_t* __restrict__ err) {
+k_scan(JobRef jr, GcMeta* meta, uint64_t* offs, uint64_t* totals, uint32_t* err) {
   __shared__ uint64_t warp_sums[kScanThreads / 32];
+  next_may_start();
+  wait_before(meta);
   const int j = blockIdx.x;
   const Job& J = job_at(jr, j);
   const int G = elem_size(J.dtype);
@@ -2205,12 +2232,12 @@ __device__ void write_header(const Job& J, uint64_t total) {
 
 template <int DTS, bool S2>
 __global__ void __launch_bounds__(kPackThreads, 2)
-k_pack(JobRef jr, uint64_t nchunks_total, const uint32_t* __restrict__ codes,
-       const uint8_t* __restrict__ tabs, const GcMeta* __restrict__ meta,
-       const uint64_t* __restrict__ offs, const uint64_t* __restrict__ totals) {
+k_pack(JobRef jr, uint64_t nchunks_total, const uint32_t* codes, const uint8_t* tabs,
+       const GcMeta* meta, const uint64_t* offs, const uint64_t* totals) {
   __shared__ PackSmem S;
   extern __shared__ uint32_t slots[];  // kPackSlotWords
   const int tid = threadIdx.x;
+  wait_before(codes, tabs, meta, offs, totals);
   if (blockIdx.x >= nchunks_total) {  // header CTAs
     const int j = (int)(blockIdx.x - nchunks_total);
     const Job& J = job_at(jr, j);
@@ -2470,6 +2497,24 @@ static JobRef make_ref(const Job* d_jobs, int njobs, const Job* h_one) {
   return r;
 }
 
+// Launch as a programmatic dependent of the kernel before it on the stream, which
+// must be the encoder's (another predecessor is simply waited for).
+template <class... KA, class... A>
+static cudaError_t launch_after(void (*kern)(KA...), unsigned grid, unsigned threads, int smem,
+                                cudaStream_t st, A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, KA(args)...);
+}
+
 // Launch k_hist, k_build and k_scan.  d_jobs is a device table of njobs jobs,
 // unless njobs == 1 and h_one is given (then the job is passed by value).
 template <class K>
@@ -2508,8 +2553,11 @@ cudaError_t launch_encode_analyse_ex(const Job* d_jobs, const Job* h_one, int nj
     if (ea != cudaSuccess) return ea;
     kh<<<(unsigned)nchunks_total, threads, hs, st>>>(r, s.hist, s.zsyms);
     unsigned nb = (unsigned)((ngc_total + kBuildWarps - 1) / kBuildWarps);
-    k_build<<<nb, kBuildWarps * 32, 0, st>>>(r, ngc_total, s.hist, s.zsyms, s.codes, s.tabs,
-                                             s.meta);
+    cudaError_t e = launch_after(k_build, nb, kBuildWarps * 32, 0, st, r, ngc_total, s.hist,
+                                 s.zsyms, s.codes, s.tabs, s.meta);
+    if (e != cudaSuccess) return e;
+    return launch_after(k_scan, (unsigned)njobs, kScanThreads, 0, st, r, s.meta, s.offs, s.totals,
+                        d_err);
   }
   k_scan<<<njobs, kScanThreads, 0, st>>>(r, s.meta, s.offs, s.totals, d_err);
   return cudaGetLastError();
@@ -2533,9 +2581,8 @@ cudaError_t launch_encode_pack_ex(const Job* d_jobs, const Job* h_one, int njobs
   const int ps = (int)(kPackSlotWords * 4);
   const cudaError_t ea = prepare_kernel(reinterpret_cast<const void*>(kp), ps);
   if (ea != cudaSuccess) return ea;
-  kp<<<(unsigned)(nchunks_total + njobs), kPackThreads, ps, st>>>(r, nchunks_total, s.codes, s.tabs,
-                                                                s.meta, s.offs, s.totals);
-  return cudaGetLastError();
+  return launch_after(kp, (unsigned)(nchunks_total + njobs), kPackThreads, ps, st, r,
+                      nchunks_total, s.codes, s.tabs, s.meta, s.offs, s.totals);
 }
 
 bool fused_encoder_applies(int dtype, bool any_skip) {

@@ -220,6 +220,21 @@ zipnn_status zipnn_batch_compress_into_ex(
     void* const* d_outs, const size_t* out_capacities, void* d_workspace,
     size_t workspace_bytes, uint64_t* d_out_nbytes, void* cuda_stream);
 
+/* Compression into a buffer of exactly the container's size, in two calls.
+ * zipnn_compress_analyse runs every step but the packing, waits for the stream
+ * and describes the container in *out (size, lanes, ...; data NULL).  The
+ * caller points out->data at nbytes bytes of device memory (16-byte aligned)
+ * and zipnn_compress_pack, given the same input, base and workspace with
+ * the contents that the first call left, enqueues the packing.  Arguments and
+ * errors as zipnn_compress_into. */
+zipnn_status zipnn_compress_analyse(const void* d_src, const void* d_base_or_null, size_t nbytes,
+                                    int dtype, size_t chunk_bytes, uint32_t lanes,
+                                    void* d_workspace, size_t workspace_bytes, zipnn_stream* out,
+                                    void* cuda_stream);
+zipnn_status zipnn_compress_pack(const void* d_src, const void* d_base_or_null,
+                                 const zipnn_stream* s, void* d_workspace, size_t workspace_bytes,
+                                 void* cuda_stream);
+
 /* Wrap a container that is already in device memory (e.g. copied from a file)
  * as a zipnn_stream: reads and validates its 64-B header (synchronous copy of
  * 64 bytes).  The stream does not own d_data.  ECORRUPT if the header is bad. */

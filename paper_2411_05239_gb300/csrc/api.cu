@@ -365,6 +365,63 @@ extern "C" zipnn_status zipnn_batch_compress_into(
                                       d_out_nbytes, cuda_stream);
 }
 
+zipnn_status zipnn_compress_analyse(const void* d_src, const void* d_base_or_null, size_t nbytes,
+                                    int dtype, size_t chunk_bytes, uint32_t lanes,
+                                    void* d_workspace, size_t workspace_bytes, zipnn_stream* out,
+                                    void* cuda_stream) {
+  if (!out) return ZIPNN_EINVAL;
+  memset(out, 0, sizeof(*out));
+  if (lanes == 0 && dtype >= ZIPNN_BF16 && dtype <= ZIPNN_U8)
+    lanes = default_lanes_for(dtype, chunk_bytes, d_base_or_null != nullptr);
+  zipnn_status rc = check_params(dtype, nbytes, chunk_bytes, lanes);
+  if (rc) return rc;
+  if ((nbytes && !d_src) || !aligned16(d_src) || !aligned16(d_base_or_null)) return ZIPNN_EINVAL;
+  if (!d_workspace || workspace_bytes < zipnn_compress_workspace_size(nbytes, dtype, chunk_bytes))
+    return ZIPNN_ENOMEM;
+  uint32_t* err = err_word();
+  if (!err) return ZIPNN_ECUDA;
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  const uint32_t flags = d_base_or_null ? ZIPNN_FLAG_DELTA : 0u;
+  Job J = make_job(d_src, d_base_or_null, nullptr, nbytes, dtype, chunk_bytes, lanes, flags);
+  const uint64_t ngc = (uint64_t)J.n_chunks * elem_size(dtype);
+  EncodeScratch s;
+  encode_scratch_carve(d_workspace, J.n_chunks, ngc, 1, &s);
+  cudaError_t e = launch_encode_analyse_ex(nullptr, &J, 1, J.n_chunks, ngc, s, err, st, 0, -1);
+  uint64_t total = 0;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&total, s.totals, 8, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return cuda_status(e);
+  out->nbytes = total;
+  out->orig_nbytes = nbytes;
+  out->dtype = dtype;
+  out->flags = flags;
+  out->chunk_bytes = (uint32_t)chunk_bytes;
+  out->lanes = lanes;
+  out->n_chunks = J.n_chunks;
+  out->n_groups = (uint32_t)elem_size(dtype);
+  return ZIPNN_OK;
+}
+
+zipnn_status zipnn_compress_pack(const void* d_src, const void* d_base_or_null,
+                                 const zipnn_stream* s, void* d_workspace, size_t workspace_bytes,
+                                 void* cuda_stream) {
+  zipnn_status rc = check_stream(s);
+  if (rc) return rc;
+  if (((s->flags & ZIPNN_FLAG_DELTA) != 0) != (d_base_or_null != nullptr)) return ZIPNN_EINVAL;
+  if ((s->orig_nbytes && !d_src) || !aligned16(d_src) || !aligned16(d_base_or_null))
+    return ZIPNN_EINVAL;
+  if (!d_workspace ||
+      workspace_bytes < zipnn_compress_workspace_size(s->orig_nbytes, s->dtype, s->chunk_bytes))
+    return ZIPNN_ENOMEM;
+  Job J = make_job(d_src, d_base_or_null, s->data, s->orig_nbytes, s->dtype, s->chunk_bytes,
+                   s->lanes, s->flags);
+  J.out_capacity = s->nbytes;
+  EncodeScratch w;
+  encode_scratch_carve(d_workspace, J.n_chunks, (uint64_t)J.n_chunks * elem_size(s->dtype), 1, &w);
+  return cuda_status(launch_encode_pack_ex(nullptr, &J, 1, J.n_chunks, (int)s->lanes, w,
+                                           static_cast<cudaStream_t>(cuda_stream), -1));
+}
+
 static zipnn_status compress_alloc(const void* d_src, const void* d_base, size_t nbytes, int dtype,
                                    size_t chunk_bytes, zipnn_stream* out, void* cuda_stream) {
   if (!out) return ZIPNN_EINVAL;
@@ -375,44 +432,22 @@ static zipnn_status compress_alloc(const void* d_src, const void* d_base, size_t
   zipnn_status rc = check_params(dtype, nbytes, chunk_bytes, lanes);
   if (rc) return rc;
   if ((nbytes && !d_src) || !aligned16(d_src) || !aligned16(d_base)) return ZIPNN_EINVAL;
-  uint32_t* err = err_word();
-  if (!err) return ZIPNN_ECUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  Job J = make_job(d_src, d_base, nullptr, nbytes, dtype, chunk_bytes, lanes,
-                   d_base ? ZIPNN_FLAG_DELTA : 0u);
-  const uint64_t ngc = (uint64_t)J.n_chunks * elem_size(dtype);
-  const size_t ws = encode_scratch_bytes(J.n_chunks, ngc, 1);
+  const size_t ws = zipnn_compress_workspace_size(nbytes, dtype, chunk_bytes);
   void* scratch = nullptr;
   cudaError_t e = cudaMallocAsync(&scratch, ws, st);
   if (e != cudaSuccess) return cuda_status(e);
-  EncodeScratch s;
-  encode_scratch_carve(scratch, J.n_chunks, ngc, 1, &s);
-  e = launch_encode_analyse_ex(nullptr, &J, 1, J.n_chunks, ngc, s, err, st, 0, -1);
-  uint64_t total = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&total, s.totals, 8, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  void* buf = nullptr;
-  if (e == cudaSuccess) e = cudaMallocAsync(&buf, total ? total : 16, st);
-  if (e == cudaSuccess) {
-    J.dst = static_cast<uint8_t*>(buf);
-    J.out_capacity = total;
-    e = launch_encode_pack_ex(nullptr, &J, 1, J.n_chunks, (int)lanes, s, st, -1);
-  }
+  zipnn_stream s;
+  rc = zipnn_compress_analyse(d_src, d_base, nbytes, dtype, chunk_bytes, lanes, scratch, ws, &s, st);
+  if (!rc) rc = cuda_status(cudaMallocAsync(&s.data, s.nbytes ? s.nbytes : 16, st));
+  if (!rc) rc = zipnn_compress_pack(d_src, d_base, &s, scratch, ws, st);
   cudaFreeAsync(scratch, st);
-  if (e != cudaSuccess) {
-    if (buf) cudaFreeAsync(buf, st);
-    return cuda_status(e);
+  if (rc) {
+    if (s.data) cudaFreeAsync(s.data, st);
+    return rc;
   }
-  out->data = buf;
-  out->nbytes = total;
-  out->orig_nbytes = nbytes;
-  out->dtype = dtype;
-  out->flags = J.flags;
-  out->chunk_bytes = (uint32_t)chunk_bytes;
-  out->lanes = lanes;
-  out->n_chunks = J.n_chunks;
-  out->n_groups = (uint32_t)elem_size(dtype);
-  out->owned = 1;
+  s.owned = 1;
+  *out = s;
   return ZIPNN_OK;
 }
 

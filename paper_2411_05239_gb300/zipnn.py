@@ -34,6 +34,7 @@ EXPORTS = [
     "zipnn_plan_decompress", "zipnn_plan_compress", "zipnn_plan_launch", "zipnn_plan_destroy",
     "zipnn_plan_load", "zipnn_batch_compress_into_ex", "zipnn_partition_chunks",
     "zipnn_plan_decompress_range", "zipnn_stream_read",
+    "zipnn_compress_analyse", "zipnn_compress_pack",
 ]
 
 
@@ -88,6 +89,8 @@ def lib() -> ctypes.CDLL:
         "zipnn_compress_into": ([vp, vp, sz, i32, sz, u32, vp, sz, vp, sz, vp, vp], i32),
         "zipnn_stream_wrap": ([vp, sz, zsp], i32),
         "zipnn_stream_read": ([vp, sz, zsp, vp], i32),
+        "zipnn_compress_analyse": ([vp, vp, sz, i32, sz, u32, vp, sz, zsp, vp], i32),
+        "zipnn_compress_pack": ([vp, vp, zsp, vp, sz, vp], i32),
         "zipnn_decompressed_size": ([zsp, ctypes.POINTER(sz), ctypes.POINTER(i32)], i32),
         "zipnn_decompress": ([zsp, vp, vp, sz, vp], i32),
         "zipnn_batch_decompress": ([zsp, ctypes.POINTER(vp), ctypes.POINTER(vp), i32,
@@ -259,22 +262,31 @@ def compress(x: torch.Tensor, chunk_bytes: int = DEFAULT_CHUNK, lanes: int = 0,
              base: torch.Tensor | None = None, dtype: int | None = None, stream=None,
              exact: bool = True) -> Compressed:
     """Compress a CUDA tensor; the container lives in a torch-allocated buffer.
-    Reads the container's header back, whose size the exact copy needs, and
-    returns when the container is complete."""
+    Returns when the container is complete.  With exact, its size is read back
+    before it is packed, into a buffer of that size; else it is packed at once
+    into a buffer of the largest possible size."""
     code = dtype_code(x, dtype)
-    n = x.numel() * x.element_size()
-    out = torch.empty(compress_bound(n, code, chunk_bytes), dtype=torch.uint8, device=x.device)
+    L, zs, st = lib(), ZStream(), _sp(stream)
+    sp, n, src = _span(x)
     ws = torch.empty(workspace_size(n, code, chunk_bytes), dtype=torch.uint8, device=x.device)
-    compress_into(x, out, ws, None, base=base, chunk_bytes=chunk_bytes, lanes=lanes, dtype=code,
-                  stream=stream)
-    zs = ZStream()
-    _check(lib().zipnn_stream_read(out.data_ptr(), out.numel(), ctypes.byref(zs), _sp(stream)),
-           "zipnn_stream_read")
     if not exact:
+        out = torch.empty(compress_bound(n, code, chunk_bytes), dtype=torch.uint8, device=x.device)
+        compress_into(src, out, ws, None, base=base, chunk_bytes=chunk_bytes, lanes=lanes,
+                      dtype=code, stream=stream)
+        _check(L.zipnn_stream_read(out.data_ptr(), out.numel(), ctypes.byref(zs), st),
+               "zipnn_stream_read")
         return Compressed(zs, out)
-    buf = out[:zs.nbytes].clone()
+    bp, nb, b = _span(base) if base is not None else (None, n, None)
+    if nb != n:
+        raise ValueError("base size differs")
+    zp, wp, wn = ctypes.byref(zs), ws.data_ptr(), ws.numel()
+    sp = sp if n else None
+    _check(L.zipnn_compress_analyse(sp, bp, n, code, chunk_bytes, lanes, wp, wn, zp, st),
+           "zipnn_compress_analyse")
+    buf = torch.empty(zs.nbytes, dtype=torch.uint8, device=x.device)
     zs.data = buf.data_ptr()
-    torch.cuda.current_stream().synchronize()
+    _check(L.zipnn_compress_pack(sp, bp, zp, wp, wn, st), "zipnn_compress_pack")
+    (stream if stream is not None else torch.cuda.current_stream()).synchronize()
     return Compressed(zs, buf)
 
 

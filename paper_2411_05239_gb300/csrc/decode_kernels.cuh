@@ -237,9 +237,11 @@ struct Bits {
 //            it by enough that a reader that was clamped fails the end check.
 //   kRinged  in global memory through a ring of 16-B pieces in shared memory
 //            per thread, filled by asynchronous copies.  nx: word index from
-//            the payload's start.  Reading the last word of a piece requests
-//            the piece `slots` further on into its slot; pieces past the
-//            payload are zero.
+//            the payload's start.  Once per vector (refill) the pieces whose
+//            slots' last words were read since are requested; pieces past the
+//            payload are zero.  (Requested where the last word of a piece was
+//            read, some lane of nearly every lookup pair had one, and the
+//            other 31 waited: 27 instructions a symbol.)
 enum Where { kStaged, kRinged };
 template <int WH> struct Source;
 template <> struct Source<kStaged> {
@@ -251,21 +253,24 @@ template <> struct Source<kStaged> {
     return v;
   }
   __device__ __forceinline__ uint32_t index(uint32_t nx) const { return (nx - base) >> 2; }
+  template <int V> __device__ __forceinline__ void refill(uint32_t) {}
 };
 template <> struct Source<kRinged> {
   const uint8_t* pay;       // the payload (16-B aligned)
   uint32_t bs, pieces;      // its bitstream's first word, its 16-B pieces
   uint32_t ring, stride;    // this thread's slot 0, bytes from slot to slot
   uint32_t mask;            // slots - 1
+  uint32_t rq;              // the piece to request next
   __device__ __forceinline__ void request(uint32_t i) const {
     const uint32_t bytes = i < pieces ? 16u : 0u;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ring + (i & mask) * stride),
                  "l"(pay + 16ull * min(i, pieces - 1u)), "r"(bytes));
   }
   // requests the pieces from word index `word` of the bitstream on
-  __device__ __forceinline__ uint32_t at(uint32_t word) const {
+  __device__ __forceinline__ uint32_t at(uint32_t word) {
     const uint32_t nx = bs + word;
     for (uint32_t i = 0; i <= mask; i++) request((nx >> 2) + i);
+    rq = (nx >> 2) + mask + 1u;
     cp_async_commit();
     cp_async_wait<0>();
     return nx;
@@ -273,25 +278,30 @@ template <> struct Source<kRinged> {
   __device__ __forceinline__ uint32_t read(uint32_t& nx) const {
     const uint32_t v = lds32v(ring + ((nx >> 2) & mask) * stride + 4u * (nx & 3u));
     nx++;
-    if ((nx & 3u) == 0) request((nx >> 2) + mask);
     return v;
+  }
+  // a vector's V codes take at most 12 V bits: 16 of them end two pieces at most,
+  // 8 or 4 one
+  template <int V> __device__ __forceinline__ void refill(uint32_t nx) {
+#pragma unroll
+    for (int k = 0; k < (V > 8 ? 2 : 1); k++)
+      if (rq <= (nx >> 2) + mask) request(rq++);
   }
   __device__ __forceinline__ uint32_t index(uint32_t nx) const { return nx - bs; }
 };
-// Ring sizes.  A piece is requested when the reader takes the last word of the
-// piece `slots` before it, i.e. at least (4 (slots - 1) 32 - 23) / 12 symbols
-// before its first word is read (12-bit codes; a lookup pair of 24 bits passes
-// a word boundary by 23 at most): 30 symbols with 4 slots, 74 with 8.  The
-// loops close one copy group per vector and wait until at most kRingPending
-// are open, so a piece has landed kRingPending + 1 vectors after its request:
-// 24 symbols for 8-symbol vectors, 12 for FP32 (4 slots suffice), 48 for U8 (8
-// slots).
+// Ring sizes.  At the start of a vector every piece from the reader's own to
+// the one `slots` - 1 further on is requested, and the loops close one copy group
+// per vector and wait until at most kRingPending are open.  So what was requested
+// by the start of two vectors ago has landed, and a vector reads at most 3 vectors'
+// bits beyond the word that was next then: 19 words for 16-symbol vectors, 5
+// pieces ahead (8 slots), 10 words or 3 pieces for 8 symbols and less for 4
+// (4 slots).
 constexpr int kRingPending = 2;
 template <int V> constexpr uint32_t ring_slots_min() { return V > 8 ? 8u : 4u; }
 constexpr uint32_t kRingSlotsMax = 8;
 
 template <int WH>
-__device__ __forceinline__ void bits_init(Bits& r, const Source<WH>& s, uint32_t start) {
+__device__ __forceinline__ void bits_init(Bits& r, Source<WH>& s, uint32_t start) {
   r.pos = start & 31u;
   r.nx = s.at(start >> 5);
   r.w0 = s.read(r.nx);
@@ -786,7 +796,10 @@ __device__ __forceinline__ void decode_general(const Smem& S, uint32_t* err, uin
         for (int g = 0; g < G; g++)
           if ((rawm >> g) & 1u) prefetch_at<V>(rawp[g], va);
       }
-      if constexpr (WH == kRinged) {  // the pieces requested kRingPending + 1 vectors ago
+      if constexpr (WH == kRinged) {
+#pragma unroll
+        for (int g = 0; g < G; g++)
+          if ((coded >> g) & 1u) src[g].template refill<V>(r[g].nx);
         cp_async_commit();
         cp_async_wait<kRingPending>();
       }

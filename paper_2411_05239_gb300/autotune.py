@@ -1,9 +1,11 @@
-"""Autotuner for the batched codec: chunk size, sub-stream lanes, decode table
-width, decoder CTA size and persistent-grid occupancy.
+"""Autotuner for the batched codec: chunk size, sub-stream lanes, decoder CTA size
+and persistent-grid occupancy.
 
 Chunk size (64 KiB - 1 MiB) and lanes are container parameters (chosen at
-compression time, recorded in the header); table width W (10-12 bits), threads
-per CTA (128 / 256) and CTAs per SM are decoder launch parameters.  None of them changes the decoded bytes.
+compression time, recorded in the header); threads per CTA (128 / 256) and CTAs per
+SM are decoder launch parameters.  None of them changes the decoded bytes.  (The
+table width lut_bits is part of a setting but has no effect any more: tables have
+12-bit windows.)
 The tuner compresses a representative sample with each candidate chunk size,
 times the graph-captured batched decode for each decoder setting, and keeps
 the fastest decode (compression speed breaks ties).  Results are cached as JSON
@@ -21,7 +23,7 @@ import torch
 from . import zipnn as Z
 
 CHUNKS = (64 << 10, 128 << 10, 256 << 10, 512 << 10, 1 << 20)
-LUT_BITS = (10, 11, 12)
+LUT_BITS = (12,)  # one width: the others decode with the same table
 
 
 def cache_path() -> str:
@@ -92,8 +94,6 @@ def tune(sample: list[torch.Tensor], reps: int = 5, chunks=CHUNKS, lut_bits=LUT_
         pc = Z.plan_compress(bc)
         t_comp = _time(pc.launch, reps)
         for w, nt, k in [(w, nt, k) for w in lut_bits for nt in threads for k in ctas]:
-            if nt != 128 and w < 11:
-                continue  # 256-thread CTAs exist for W >= 11 only
             pd = Z.plan_decompress(cs, outs, tune=Z.tuning(threads=nt, ctas_per_sm=k, lut_bits=w))
             t_dec = _time(pd.launch, reps)
             pd.close()

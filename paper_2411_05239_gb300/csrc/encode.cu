@@ -3,11 +3,12 @@
 //   k_hist      one CTA per chunk: reads the chunk once with 16-B loads (XOR
 //               with the delta base fused in), applies the exponent-extraction /
 //               byte-grouping permutation in registers and builds one 256-bin
-//               histogram per byte group (per-warp shared-memory copies).
+//               histogram per byte group (lane-indexed shared-memory counters).
 //   k_build     one warp per group-chunk: mode decision (ZERO / CONST / RAW /
-//               HUFF), length-limited code lengths by package-merge (limit 12),
-//               canonical codes and the table bytes.  A Shannon lower bound
-//               proves RAW without building a code for incompressible groups.
+//               HUFF / SPARSE), length-limited code lengths by package-merge in
+//               registers (limit 12), canonical codes and the table bytes.  A
+//               Shannon lower bound proves RAW without building a code for
+//               incompressible groups.
 //   k_scan      one CTA per tensor: exclusive scan of the padded payload sizes
 //               (the chunk map of Sec. 5.1) and the container size.
 //   k_pack      one CTA per chunk: per-sub-stream bit counts, a CTA scan for

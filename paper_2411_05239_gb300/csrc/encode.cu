@@ -2059,8 +2059,11 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
     }
     if (lane == 31) S.wsum[wid] = uincl;
   } else if (DT == ZIPNN_FP32) {
-    for (uint32_t u = tid; whole && u < units; u += nthr)
-      whole = S.sbits[u] >= 32u && S.sbits[u] <= slot_cap * 32u;
+    // (this thread's own units: nothing has waited for the other threads yet)
+    for (uint32_t u = tid; whole && u < units; u += nthr) {
+      const uint32_t b = S.sbits[gmod(u, T) * R + gdiv(u, T)];
+      whole = b >= 32u && b <= slot_cap * 32u;
+    }
   } else {
     whole = false;
   }

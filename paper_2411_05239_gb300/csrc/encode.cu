@@ -2038,11 +2038,12 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
   if (!huff) return;
   // Pass B writes each output word of the staged groups whole (no zeroed words,
   // no atomics) when every coded group is staged and every unit fits its slot:
-  // pass_b_whole when there is one group, 32 bits or more in every unit (so that a
+  // pass_b_whole when there is one group, HUFF (a SPARSE one has its bitmap before
+  // the starts, and empty units), 32 bits or more in every unit (so that a
   // word spans at most two) and a unit per thread or FP32 (256 MiB: 229.6 us
   // against 232.7; a second copy of it costs the 16-bit kernels more in
   // registers than it gains with several units a thread), else pass_b_any
-  bool whole = sg == 0 && huff == 1u;
+  bool whole = sg == 0 && huff == 1u && sparse == 0;
   // one unit per thread (unit tid): its exclusive bit offset from a warp scan
   // before this barrier and a scan of the warp totals after it
   const bool one = R == 1 && units == (uint32_t)nthr;

@@ -22,42 +22,49 @@ struct DecodeConfig {
   uint32_t ntab, stage, ring;
 };
 
-// The stage has room for the coded payloads of the largest chunk, as a fraction
-// of it (frac64 / 64, see stage_frac64) or as a plan read it from the chunk
-// maps (stage_need), as far as the CTAs per SM of the kernel's register budget,
-// or two, still share an SM (a launch of fewer work items than that needs
-// less).  Payloads a little larger are decoded in slices.  Payloads much larger
-// than that (1 MiB chunks: one CTA per SM) and all of U8's are not staged: the
-// stage then holds the readers' rings, kRingSlotsMax pieces of 16 B per thread.
-// Always room, with the raw-word rings behind the stage, for the tables of
-// every coded group after the first ntab.
+// The stage is meant to hold the coded payloads of the largest chunk: a fraction
+// of it (frac64 / 64, see stage_frac64) or what a plan read from the chunk maps
+// (stage_need).  It takes all the shared memory that the most CTAs per SM with
+// room for that leave it: as many as the kernel's registers allow, at least two of
+// 256 threads (a launch of fewer work items than that: one).  Payloads that do not
+// fit are decoded in slices, so there is always room, with the raw-word rings
+// behind the stage, for the tables of every coded group after the first ntab and
+// for the least slice.  Where payloads much larger than the stage are expected (1 MiB
+// chunks: one CTA per SM) or there is no such room, and for U8, they are not staged: the
+// stage holds the readers' rings, kRingSlotsMax pieces of 16 B per thread.
 DecodeConfig decode_config(const DecodeShape& sh, int threads, uint64_t items_per_sm) {
   DecodeConfig c;
   const uint32_t per_cta = kSmReserve + kStaticReserve;
+  const bool fp32 = sh.family == ZIPNN_FP32;
   c.kind = sh.delta ? kDeltas : kWeights;
-  c.ntab = sh.delta && sh.max_groups > 1 ? 2u : 1u;
-  c.ring = sh.family == ZIPNN_FP32 && !sh.delta ? kRingBytes * (uint32_t)threads : 0u;
+  c.ntab = c.kind == kDeltas && sh.max_groups > 1 ? 2u : 1u;
+  c.ring = fp32 && c.kind == kWeights ? kRingBytes * (uint32_t)threads : 0u;
   const uint32_t tabs =
       sh.max_groups > (int)c.ntab ? (uint32_t)(sh.max_groups - (int)c.ntab) * kLutBytes : 0u;
-  const uint32_t scale = 256u / (uint32_t)threads;
-  auto cap = [&](uint64_t ctas) -> uint64_t {
-    if (ctas > items_per_sm) ctas = items_per_sm ? items_per_sm : 1;
+  auto cap = [&](uint32_t ctas) -> uint32_t {  // the stage that leaves `ctas` per SM
     return kSmPerSm / ctas - per_cta - c.ntab * kLutBytes - c.ring;
   };
-  const uint64_t cap2 = cap(2u * scale);
-  uint64_t want = sh.stage_need ? sh.stage_need : sh.max_chunk * (uint64_t)sh.frac64 / 64 + 1024;
-  // the least slice: the longest sub-stream of every group that the codes
-  // allow (12 bits a symbol)
-  const uint64_t least = (sh.max_chunk / sh.min_lanes * 3 / 2 + 128 * (uint64_t)sh.max_groups) + tabs;
-  if (sh.family == ZIPNN_U8 || (want > cap2 + cap2 / 8 && !sh.stage_need) || least > cap2) {
+  const uint64_t want =
+      sh.stage_need ? sh.stage_need : sh.max_chunk * (uint64_t)sh.frac64 / 64 + 1024;
+  // the least slice: of every group the longest sub-stream that the codes allow (12
+  // bits a symbol), and what its pieces are rounded to
+  const uint64_t vecs = (sh.max_chunk / 16 + sh.min_lanes - 1) / sh.min_lanes;
+  const uint64_t slice = tabs + vecs * 24 + 192 * (uint64_t)sh.max_groups;
+  const uint32_t two = 2u * (256u / (uint32_t)threads);
+  const uint32_t least = items_per_sm >= two ? two : (items_per_sm ? (uint32_t)items_per_sm : 1u);
+  // (the register budgets of the kernels, see kernel_of)
+  uint32_t ctas = threads == 256 && (!fp32 || c.kind == kWeights) ? 3u : two;
+  while (ctas > least && cap(ctas) < want) ctas--;
+  while (ctas > 1u && cap(ctas) + c.ring < slice) ctas--;
+  const uint64_t room = cap(ctas);
+  if (sh.family == ZIPNN_U8 || (want > room + room / 8 && !sh.stage_need) ||
+      room + c.ring < slice) {
     c.kind = kRings;
     c.ring = 0;
-    want = kRingSlotsMax * 16u * (uint64_t)threads + tabs;
+    c.stage = kRingSlotsMax * 16u * (uint32_t)threads + tabs;
   } else {
-    if (want > cap2) want = cap2;
-    if (want + c.ring < least + 4096u) want = least + 4096u - c.ring;
+    c.stage = (uint32_t)room;
   }
-  c.stage = ((uint32_t)want + 127u) & ~127u;
   return c;
 }
 

@@ -31,12 +31,15 @@ struct DecodeConfig {
 // behind the stage, for the tables of every coded group after the first ntab and
 // for the least slice.  Where payloads much larger than the stage are expected (1 MiB
 // chunks: one CTA per SM) or there is no such room, and for U8, they are not staged: the
-// stage holds the readers' rings, kRingSlotsMax pieces of 16 B per thread.
+// stage holds the readers' rings, kRingSlotsMax pieces of 16 B per thread.  FP32 plans
+// most of whose chunks do not take the weight loop (`general`) take the kernel for
+// deltas, which has the general loop alone, while their payloads fit its stage (256 MiB
+// pruned to 10%: 267 us, by rings 832), else the rings (16 values: 512 us; by slices 667).
 DecodeConfig decode_config(const DecodeShape& sh, int threads, uint64_t items_per_sm) {
   DecodeConfig c;
   const uint32_t per_cta = kSmReserve + kStaticReserve;
   const bool fp32 = sh.family == ZIPNN_FP32;
-  c.kind = sh.delta ? kDeltas : kWeights;
+  c.kind = sh.delta || sh.general ? kDeltas : kWeights;
   c.ntab = c.kind == kDeltas && sh.max_groups > 1 ? 2u : 1u;
   c.ring = fp32 && c.kind == kWeights ? kRingBytes * (uint32_t)threads : 0u;
   const uint32_t tabs =
@@ -46,19 +49,23 @@ DecodeConfig decode_config(const DecodeShape& sh, int threads, uint64_t items_pe
   };
   const uint64_t want =
       sh.stage_need ? sh.stage_need : sh.max_chunk * (uint64_t)sh.frac64 / 64 + 1024;
-  // the least slice: of every group the longest sub-stream that the codes allow (12
-  // bits a symbol), and what its pieces are rounded to
+  // the least slice: of every coded group the longest sub-stream that the codes allow
+  // (12 bits a symbol), the bitmap, and what its pieces are rounded to.  FP32 weights
+  // slice chunks of one HUFF group only, which need no other table (kReadsDirect).
   const uint64_t vecs = (sh.max_chunk / 16 + sh.min_lanes - 1) / sh.min_lanes;
-  const uint64_t slice = tabs + vecs * 24 + 192 * (uint64_t)sh.max_groups;
+  const uint64_t slice =
+      fp32 && c.kind == kWeights
+          ? vecs * 6 + 192
+          : tabs + vecs * 24 + (sh.max_chunk / 128 + 192) * (uint64_t)sh.max_groups;
   const uint32_t two = 2u * (256u / (uint32_t)threads);
   const uint32_t least = items_per_sm >= two ? two : (items_per_sm ? (uint32_t)items_per_sm : 1u);
   // (the register budgets of the kernels, see kernel_of)
   uint32_t ctas = threads == 256 && (!fp32 || c.kind == kWeights) ? 3u : two;
   while (ctas > least && cap(ctas) < want) ctas--;
-  while (ctas > 1u && cap(ctas) + c.ring < slice) ctas--;
+  while (ctas > 1u && (cap(ctas) < slice || cap(ctas) + c.ring < tabs)) ctas--;
   const uint64_t room = cap(ctas);
-  if (sh.family == ZIPNN_U8 || (want > room + room / 8 && !sh.stage_need) ||
-      room + c.ring < slice) {
+  const bool over = want > room + (sh.general ? 0 : room / 8);
+  if (sh.family == ZIPNN_U8 || (over && (!sh.stage_need || sh.general)) || room < slice) {
     c.kind = kRings;
     c.ring = 0;
     c.stage = kRingSlotsMax * 16u * (uint32_t)threads + tabs;

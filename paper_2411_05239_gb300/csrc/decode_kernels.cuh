@@ -147,7 +147,8 @@ struct ChunkInfo {
   uint32_t pairs;           // bit g: its table holds pairs
   uint32_t stage;           // shared-window address of the stage behind the tables,
   uint32_t stage_bytes;     // its size,
-  uint32_t sliced;          // and whether the payloads only fit it in slices
+  uint32_t sliced;          // whether the payloads only fit it in slices,
+  uint32_t direct;          // or stay in global memory
   uint32_t ring_slots;      // kRinged: slots of the readers' rings at `stage`,
   uint32_t ring_threads;    // and the threads that have one
   uint32_t bad;             // 1: bad map entry or table, 2: a bulk copy timed out
@@ -242,7 +243,9 @@ struct Bits {
 //            payload are zero.  (Requested where the last word of a piece was
 //            read, some lane of nearly every lookup pair had one, and the
 //            other 31 waited: 27 instructions a symbol.)
-enum Where { kStaged, kRinged };
+//   kDirect  in global memory, word by word; zero bits past the last one.  nx: word
+//            index.
+enum Where { kStaged, kRinged, kDirect };
 template <int WH> struct Source;
 template <> struct Source<kStaged> {
   uint32_t base, end;
@@ -288,6 +291,18 @@ template <> struct Source<kRinged> {
       if (rq <= (nx >> 2) + mask) request(rq++);
   }
   __device__ __forceinline__ uint32_t index(uint32_t nx) const { return nx - bs; }
+};
+template <> struct Source<kDirect> {
+  const uint8_t* words;
+  uint32_t n;
+  __device__ __forceinline__ uint32_t at(uint32_t word) const { return word; }
+  __device__ __forceinline__ uint32_t read(uint32_t& nx) const {
+    const uint32_t v = nx < n ? rd_u32(words + 4ull * nx) : 0u;
+    nx++;
+    return v;
+  }
+  __device__ __forceinline__ uint32_t index(uint32_t nx) const { return nx; }
+  template <int V> __device__ __forceinline__ void refill(uint32_t) {}
 };
 // Ring sizes.  At the start of a vector every piece from the reader's own to
 // the one `slots` - 1 further on is requested, and the loops close one copy group
@@ -746,6 +761,9 @@ __device__ __forceinline__ void decode_general(const Smem& S, uint32_t* err, uin
     if constexpr (WH == kStaged) {
       src[g].base = CI.at_words[g];
       src[g].end = CI.end[g];
+    } else if constexpr (WH == kDirect) {
+      src[g].words = rawp[g] + CI.bs[g];
+      src[g].n = CI.nwords[g];
     } else {
       const uint32_t slots = CI.ring_slots;
       src[g].pay = rawp[g];
@@ -861,7 +879,7 @@ __device__ __forceinline__ void decode_general(const Smem& S, uint32_t* err, uin
 // Set-up of the next item (S.job, S.chunk, S.part, S.entry) by warp 0: its
 // record, placement of tables and payloads, the bulk copies, table bytes and
 // canonical limits, into S.it, S.ci and S.tab.
-template <int DT, int NT, bool RINGED>
+template <int DT, int NT, bool RINGED, bool DIRECT>
 __device__ __forceinline__ void setup_item(Smem& S, uint32_t parts, uint32_t lut0, uint32_t ntab,
                                            uint32_t stage_cap, uint32_t ring_bytes, uint64_t* bar,
                                            uint32_t extra_tx) {
@@ -923,6 +941,8 @@ __device__ __forceinline__ void setup_item(Smem& S, uint32_t parts, uint32_t lut
     total += s;
   }
   const bool fits = total + 32u <= room;
+  // (DIRECT: what does not take the weight loop is read from global memory)
+  const bool direct = DIRECT && !__shfl_sync(0xffffffffu, coded == 1u && mode == kHuff, 0);
   const uint32_t at = stage0 + extra + (uint32_t)before;
   if (lane < (uint32_t)G) {
     const uint32_t k = (uint32_t)__popc(coded & ((1u << lane) - 1u));
@@ -932,7 +952,7 @@ __device__ __forceinline__ void setup_item(Smem& S, uint32_t parts, uint32_t lut
     CI.payload[lane] = pay;
     CI.lut[lane] = k < ntab ? lut0 + k * kLutBytes : stage0 + (k - ntab) * kLutBytes;
   }
-  const bool copy = !RINGED && fits && nhuff;
+  const bool copy = !RINGED && fits && nhuff && !direct;
   if (copy) {
     if (lane == 0) mbar_expect_tx(bar, (uint32_t)total + extra_tx);
     __syncwarp();
@@ -1020,7 +1040,8 @@ __device__ __forceinline__ void setup_item(Smem& S, uint32_t parts, uint32_t lut
     CI.pairs = pairs;
     CI.stage = stage0 + extra;
     CI.stage_bytes = copy ? (uint32_t)total : (RINGED ? 0u : room);
-    CI.sliced = !RINGED && nhuff && !fits;
+    CI.sliced = !RINGED && nhuff && !fits && !direct;
+    if (DIRECT) CI.direct = direct;
     CI.ring_slots = slots;
     CI.ring_threads = nhuff ? threads : (uint32_t)NT;
     CI.bad = bad ? 1u : 0u;
@@ -1030,10 +1051,11 @@ __device__ __forceinline__ void setup_item(Smem& S, uint32_t parts, uint32_t lut
 // Payloads that do not fit the stage (FP16 holding BF16 values, 1 MiB chunks):
 // the sub-streams from t_a on are decoded slice by slice, each with its own
 // part of the start-bit tables and bitstreams in the stage (the sub-streams
-// follow one another in the bitstream).  Thread 0: picks the slice [t_a, t_b),
-// as many sub-streams as fit of the rest, its half, its quarter ..., requests
-// its bytes and sets the addresses; returns t_b, or 0 if not one fits.  (A launch whose sub-streams
-// are too long for one to fit takes the kernels with rings.)
+// follow one another in the bitstream) and with the bitmaps of SPARSE groups.
+// Thread 0: picks the slice [t_a, t_b), as many sub-streams as fit of the rest, its
+// half, its quarter ..., requests its bytes and sets the addresses; returns t_b, or 0
+// if not one fits (a launch has a stage for the longest one that a valid container
+// can hold).
 template <int DT>
 __device__ __noinline__ uint32_t stage_slice(Smem& S, uint32_t t_a, uint64_t* bar) {
   constexpr int G = Traits<DT>::G;
@@ -1156,11 +1178,17 @@ __device__ __forceinline__ void second_codes(const Smem& S) {
 // general loop alone: sharing the kernel costs it registers), kRings for
 // launches whose payloads do not fit the stage (the general loop over rings).
 enum Kind { kWeights, kDeltas, kRings };
+// FP32 weights: the tables of four coded groups leave next to no stage where three CTAs
+// share an SM, so chunks that do not take the weight loop are read from global
+// memory.  (256 MiB of 16 values, all groups coded: 647 us; by slices of a few
+// sub-streams 3840.  With both forms of the general loop the kernel spills and this
+// takes 967; plans have another kernel for such tensors, see decode_config.)
+template <int DT, int KIND> constexpr bool kReadsDirect = DT == ZIPNN_FP32 && KIND == kWeights;
 
-template <int DT, int NT>
+template <int DT, int KIND, int NT>
 __device__ __noinline__ void decode_general_ool(const Smem& S, uint32_t* err, uint32_t t_a,
                                                 uint32_t t_b) {
-  decode_general<DT, kStaged, NT>(S, err, t_a, t_b);
+  decode_general<DT, kReadsDirect<DT, KIND> ? kDirect : kStaged, NT>(S, err, t_a, t_b);
 }
 
 // Decode sub-streams [t_a, t_b) of the current item.
@@ -1179,7 +1207,7 @@ __device__ __forceinline__ void decode_range(const Smem& S, uint32_t lut0, uint3
         return;
       }
     }
-    if constexpr (KIND == kWeights) decode_general_ool<DT, NT>(S, err, t_a, t_b);
+    if constexpr (KIND == kWeights) decode_general_ool<DT, KIND, NT>(S, err, t_a, t_b);
     else decode_general<DT, kStaged, NT>(S, err, t_a, t_b);
   }
 }
@@ -1276,7 +1304,8 @@ k_decode(JobRef jr, uint64_t nchunks_total, uint32_t* __restrict__ err,
     if (tid < 32) {
       __syncwarp();
       if (!S.last)
-        setup_item<DT, NT, KIND == kRings>(S, parts, lut0, ntab, stage_cap, ring_bytes, &bar, extra_tx);
+        setup_item<DT, NT, KIND == kRings, kReadsDirect<DT, KIND>>(S, parts, lut0, ntab, stage_cap,
+                                                                   ring_bytes, &bar, extra_tx);
     } else if (!S.last) {
       prefetch_window<DT, NT>(S, parts, pf_bytes);
     }
@@ -1284,7 +1313,8 @@ k_decode(JobRef jr, uint64_t nchunks_total, uint32_t* __restrict__ err,
     if (S.last) break;
     const bool rejected = S.ci.bad != 0;
     const bool sliced = KIND != kRings && S.ci.sliced;
-    const bool copied = KIND != kRings && S.ci.coded && !sliced;
+    const bool copied = KIND != kRings && S.ci.coded && !sliced &&
+                        !(kReadsDirect<DT, KIND> && S.ci.direct);
     uint64_t item = 0;
     if (tid == 0) item = draw(iter);  // (needed after the next barrier)
     if (!rejected && S.ci.coded) first_codes<DT, NT>(S);

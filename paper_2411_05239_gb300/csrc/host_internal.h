@@ -76,6 +76,7 @@ struct DecodeShape {
   bool delta = false;      // some job has a base
   int frac64 = 0;          // payload bytes as a fraction of the largest chunk (stage_frac64)
   uint32_t stage_need = 0; // stage bytes measured from the chunk maps (0 = use frac64)
+  bool general = false;    // FP32: most chunks do not take the weight loop, by the maps
   void add(int dtype, uint32_t flags, uint32_t chunk_bytes, uint32_t lanes) {
     const int g = elem_size(dtype), q = stage_frac64(dtype, flags);
     family = dtype_family(dtype);

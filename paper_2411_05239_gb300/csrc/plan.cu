@@ -33,18 +33,24 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 // What a decode launch needs, read from its containers' chunk maps: per chunk
 // the shared-memory stage that holds its coded (HUFF / SPARSE) payloads, 16-B
-// padded, plus 32 B and the table of every coded group after the first (the
-// decoder's staging rule).
+// padded, plus 32 B and the tables of its coded groups past those that have slots
+// (the decoder's staging rule).
 struct MapNeed {
   uint64_t max_stage = 0;  // largest per-chunk need
   uint64_t chunks = 0;     // chunks seen
   uint64_t over = 0;       // chunks whose need exceeds the default stage
 };
+// Of FP32 weights the chunks of one HUFF group in front, and the others, which the
+// kernel for weights does not stage.
+struct MapNeeds {
+  MapNeed weights, others;
+};
 
-void add_map_need(const uint8_t* map, uint32_t n_chunks, uint32_t G, uint64_t dflt, MapNeed* nd) {
+void add_map_need(const uint8_t* map, uint32_t n_chunks, uint32_t G, uint64_t dflt, MapNeeds* nd) {
   for (uint32_t c = 0; c < n_chunks; c++) {
     uint64_t used = 0;
     uint32_t ncoded = 0;
+    bool first = false;
     for (uint32_t g = 0; g < G; g++) {
       const uint8_t* e = map + ((uint64_t)c * G + g) * kEntryBytes;
       uint32_t size;
@@ -53,23 +59,42 @@ void add_map_need(const uint8_t* map, uint32_t n_chunks, uint32_t G, uint64_t df
       if (mode == kHuff || mode == kSparse) {
         used += align_up(size, 16);
         ncoded++;
+        if (g == 0) first = mode == kHuff;
       }
     }
-    nd->chunks++;
+    const bool other = G == 4 && ncoded && !(ncoded == 1 && first);
+    MapNeed& m = other ? nd->others : nd->weights;
+    m.chunks++;
     if (ncoded) {
-      const uint64_t need = used + 32 + (uint64_t)(ncoded - 1) * 4u * kLutSize;
-      if (need > nd->max_stage) nd->max_stage = need;
-      if (need > dflt) nd->over++;
+      const uint32_t slots = other ? 2 : 1;
+      const uint64_t need =
+          used + 32 + (ncoded > slots ? (uint64_t)(ncoded - slots) * 4u * kLutSize : 0u);
+      if (need > m.max_stage) m.max_stage = need;
+      if (need > dflt) m.over++;
     }
   }
 }
 
 // The stage a plan asks for: 0 (the launcher's default rule) while the default
 // stage holds the payloads of at least 99% of the chunks, else the largest
-// need (which the launcher takes as far as two CTAs still share an SM).
-uint32_t planned_stage(const MapNeed& nd) {
-  if (nd.over * 100 <= nd.chunks) return 0;
-  return (uint32_t)(nd.max_stage > 0xFFFFFFFFull ? 0xFFFFFFFFull : nd.max_stage);
+// need (which the launcher takes as far as two CTAs still share an SM).  FP32 plans
+// most of whose chunks do not take the weight loop ask for the others' need.
+void planned_stage(const MapNeeds& nd, DecodeShape* sh) {
+  auto need = [](const MapNeed& m) -> uint32_t {
+    return (uint32_t)(m.max_stage > 0xFFFFFFFFull ? 0xFFFFFFFFull : m.max_stage);
+  };
+  if (!sh->delta && nd.others.chunks > nd.weights.chunks) {
+    sh->general = true;
+    sh->stage_need = std::max(need(nd.others), need(nd.weights));
+    return;
+  }
+  MapNeed m = nd.weights;
+  if (sh->delta) {
+    m.max_stage = std::max(m.max_stage, nd.others.max_stage);
+    m.chunks += nd.others.chunks;
+    m.over += nd.others.over;
+  }
+  sh->stage_need = m.over * 100 <= m.chunks ? 0 : need(m);
 }
 
 zipnn_status fail(zipnn_plan* p, cudaError_t e) {
@@ -159,7 +184,7 @@ static zipnn_status plan_decode_range(const zipnn_stream* streams, const void* c
   std::vector<uint8_t> mb;
   for (int k = 0; k < ngroups; k++) {
     DecodeGroup& G = groups[k];
-    MapNeed nd;
+    MapNeeds nd;
     const uint64_t dflt = G.shape.max_chunk * (uint64_t)G.shape.frac64 / 64 + 1024;
     for (int i = G.first; i < G.first + G.count; i++) {
       const Job& J = jobs[(size_t)i];
@@ -174,7 +199,7 @@ static zipnn_status plan_decode_range(const zipnn_stream* streams, const void* c
       add_map_need(mb.data() + (uint64_t)J.chunk0 * ng * kEntryBytes, (uint32_t)(end - J.chunk_begin),
                    ng, dflt, &nd);
     }
-    G.shape.stage_need = planned_stage(nd);
+    planned_stage(nd, &G.shape);
   }
   uint32_t* err = plan_err_word();
   if (!err) return ZIPNN_ECUDA;
@@ -366,7 +391,7 @@ zipnn_status zipnn_plan_load(const zipnn_stream* streams, const void* const* h_c
     std::copy(part.begin(), part.end(), jobs.begin() + a);
     for (int f = 0; f < sg.n; f++) {
       DecodeGroup& G = sg.groups[f];
-      MapNeed nd;
+      MapNeeds nd;
       const uint64_t dflt = G.shape.max_chunk * (uint64_t)G.shape.frac64 / 64 + 1024;
       for (int i = a; i < b; i++) {
         const zipnn_stream* s = &streams[i];
@@ -376,7 +401,7 @@ zipnn_status zipnn_plan_load(const zipnn_stream* streams, const void* const* h_c
         add_map_need(static_cast<const uint8_t*>(h_containers[i]) + kHdrBytes, s->n_chunks,
                      s->n_groups, dflt, &nd);
       }
-      G.shape.stage_need = planned_stage(nd);
+      planned_stage(nd, &G.shape);
     }
   }
   uint32_t* err = plan_err_word();

@@ -67,3 +67,96 @@ def test_sparse_beside_raw(kind, live, lanes):
     Z.decompress(c, out)
     Z.sync_status()
     assert torch.equal(out.view(torch.uint8), t.view(torch.uint8))
+
+
+# -- FP32 with several SPARSE groups, whose bitmaps and tables leave little stage
+
+
+def fp32_delta(vectors: int, live: float, seed: int) -> tuple[np.ndarray, np.ndarray]:
+    """(next, base) bytes of FP32 weights of which a share of the 16-byte vectors
+    changed, in every byte."""
+    g = np.random.default_rng(seed)
+    base = (g.standard_normal(vectors * 4) * 0.02).astype(np.float32).view(np.uint8)
+    return base ^ pruned("fp32", vectors, live, seed + 1), base
+
+
+def decode_every_way(c, want: torch.Tensor, base: torch.Tensor | None = None) -> None:
+    from paper_2411_05239_gb300 import zipnn as Z
+    out = torch.zeros_like(want)
+
+    def check(what):
+        Z.sync_status()
+        assert torch.equal(out.view(torch.uint8), want.view(torch.uint8)), what
+        out.zero_()
+
+    Z.decompress(c, out, base=base)
+    check("alone")
+    bases = None if base is None else [base]
+    for tune in (None, Z.tuning(threads=128), Z.tuning(threads=256), Z.tuning(parts=4)):
+        Z.batch_decompress([c], [out], bases=bases, tune=tune)
+        check("batch")
+        p = Z.plan_decompress([c], [out], bases=bases, tune=tune)
+        p.launch()
+        check("plan")
+        p.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("chunk", [65536, 131072, 262144, 524288])
+@pytest.mark.parametrize("live", [0.02, 0.05])
+@pytest.mark.parametrize("delta", [False, True])
+def test_fp32_with_four_sparse_groups(chunk, live, delta):
+    from paper_2411_05239_gb300 import zipnn as Z
+    v = 5 * chunk // 16 + 333
+    x, b = fp32_delta(v, live, 700) if delta else (pruned("fp32", v, live, 700), None)
+    lanes = O.default_lanes(O.FP32, chunk, delta)
+    want = O.delta(x, b, O.FP32, chunk, lanes) if delta else O.compress(x, O.FP32, chunk, lanes)
+    assert modes(want)[0] == (SPARSE,) * 4
+    t = torch.from_numpy(x).cuda().view(torch.float32)
+    base = None if b is None else torch.from_numpy(b).cuda().view(torch.float32)
+    c = Z.compress(t, chunk_bytes=chunk, base=base)
+    assert c.to_bytes() == want
+    decode_every_way(c, t, base)
+
+
+@pytest.mark.gpu
+def test_sparse_chunks_among_weights():
+    """One tensor whose chunks are weights but for one in 200 (a plan then keeps the
+    kernel and the stage for weights), and one with every mix of groups."""
+    from paper_2411_05239_gb300 import zipnn as Z
+    g = np.random.default_rng(701)
+    n = 65536 // 4
+    x = (g.standard_normal(200 * n) * 0.02).astype(np.float32)
+    x[77 * n:78 * n] = pruned("fp32", n // 4, 0.05, 702).view(np.float32)
+    t = torch.from_numpy(x).cuda()
+    c = Z.compress(t, chunk_bytes=65536)
+    assert [m for m in modes(c.to_bytes()) if m != (1, 0, 0, 0)] == [(SPARSE,) * 4]
+    decode_every_way(c, t)
+    v = np.zeros((16, n, 4), np.uint8)
+    for k in range(16):                      # group sets coded and raw
+        for byte in range(4):
+            v[k, :, byte] = (g.integers(0, 4, n) if k >> byte & 1 else g.integers(0, 256, n))
+    t = torch.from_numpy(v.reshape(-1)).cuda().view(torch.float32)
+    c = Z.compress(t, chunk_bytes=65536)
+    assert c.to_bytes() == O.compress(v.reshape(-1), O.FP32, 65536, Z.default_lanes(O.FP32, 65536))
+    decode_every_way(c, t)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("chunk", [1 << 20, 8 << 20, 16 << 20])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_deltas_in_large_chunks(chunk, dtype):
+    """Bitmaps of more than a stage, of two and of four groups."""
+    from paper_2411_05239_gb300 import zipnn as Z
+    g = np.random.default_rng(703)
+    v = chunk // 16 + 1251
+    low = [127, 3] if dtype == torch.bfloat16 else [63, 63, 63, 3]    # bits that change, by byte
+    x = g.integers(0, 256, (v, 16), dtype=np.uint8) & np.resize(np.array(low, np.uint8), 16)
+    x[g.random(v) >= 0.3] = 0
+    base = torch.from_numpy(pruned("bf16", v, 1.0, 704)).cuda()
+    t = (base ^ torch.from_numpy(x.reshape(-1)).cuda()).view(dtype)
+    base = base.view(dtype)
+    c = Z.delta(t, base, chunk_bytes=chunk)
+    m = modes(c.to_bytes())[0]
+    assert m == (SPARSE,) * len(m)
+    decode_every_way(c, t, base)

@@ -361,7 +361,9 @@ size_t or_bound(size_t nbytes, int dtype, size_t chunk_bytes) {
  * Returns the payload size written to out (capacity >= m + 1100 bytes).     */
 typedef struct { int mode; int value; size_t size; } or_group_result;
 
-/* table bytes: BITS[12] then the symbols ordered by (length, symbol) */
+/* table bytes: BITS[12] then the symbols ordered by (length, symbol).  The one count
+ * that does not fit its byte, 256 codes of 8 bits (SPARSE over uniform bytes), is
+ * stored as 0: twelve zero counts and the symbols 0..255 mean that code.    */
 static size_t write_table(const uint8_t* len, uint8_t* out) {
     int k = 12;
     for (int l = 1; l <= OR_MAXLEN; l++) {
@@ -623,6 +625,11 @@ static int decode_group(const uint8_t* p, size_t size, size_t m, uint32_t T, uin
     uint32_t count[OR_MAXLEN + 1] = {0};
     int nz = 0;
     for (int l = 1; l <= OR_MAXLEN; l++) { count[l] = p[l - 1]; nz += (int)count[l]; }
+    if (nz == 0 && size >= 268) {               /* 256 codes of 8 bits, see write_table */
+        int k = 0;
+        while (k < 256 && p[12 + k] == k) k++;
+        if (k == 256) count[8] = (uint32_t)(nz = 256);
+    }
     if (nz < 2 || nz > 256) return OR_ECORRUPT;
     uint64_t kraft = 0;
     for (int l = 1; l <= OR_MAXLEN; l++) kraft += (uint64_t)count[l] << (OR_MAXLEN - l);

@@ -981,7 +981,12 @@ __device__ __forceinline__ void setup_item(Smem& S, uint32_t parts, uint32_t lut
     if (i2 < 68u) t.words[i2] = b2;
     const uint32_t cword = __shfl_sync(0xffffffffu, b0, ((lane - 1u) >> 2) & 3u);
     const bool is_len = lane >= 1u && lane <= (uint32_t)kMaxLen;
-    const uint32_t cl = is_len ? (cword >> (8u * ((lane - 1u) & 3u))) & 0xFFu : 0u;
+    // 256 codes of 8 bits, whose count is stored as 0: twelve zeros, symbols 0..255
+    auto flat = [](uint32_t i) { return i < 3u ? 0u : 0x03020100u + 0x04040404u * (i - 3u); };
+    const bool all8 = __all_sync(0xffffffffu, b0 == flat(lane) && b1 == flat(i1) &&
+                                                  (i2 > 66u || b2 == flat(i2)));
+    const uint32_t cl = all8 && lane == 8u ? 256u
+                        : is_len ? (cword >> (8u * ((lane - 1u) & 3u))) & 0xFFu : 0u;
     const uint32_t A = is_len ? cl << (kMaxLen - lane) : 0u;
     uint32_t lim = A, idx = cl;
 #pragma unroll

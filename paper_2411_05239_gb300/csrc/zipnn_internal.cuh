@@ -7,7 +7,9 @@
 // bytes, u8 mode, u8 value, u16 zero.
 // HUFF payload: u8 count of codes per length 1..12, the symbols ordered by
 // (length, symbol), zero pad to 4 B, u32 start bit of sub-streams 1..T-1, then
-// the bitstream as u32 words whose most significant bit comes first.
+// the bitstream as u32 words whose most significant bit comes first.  The one
+// count that does not fit its byte, 256 codes of 8 bits (SPARSE groups of uniform
+// bytes), is stored as 0: twelve zero counts and the symbols 0..255 mean that code.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>

@@ -160,3 +160,53 @@ def test_deltas_in_large_chunks(chunk, dtype):
     m = modes(c.to_bytes())[0]
     assert m == (SPARSE,) * len(m)
     decode_every_way(c, t, base)
+
+
+# -- 256 codes of 8 bits: uniform bytes in the live vectors
+
+
+def flat_groups(s: bytes) -> list[int]:
+    """Payload offsets of the coded groups whose twelve counts are stored as 0."""
+    G, nch = struct.unpack_from("<II", s, 24)
+    P = struct.unpack_from("<Q", s, 32)[0]
+    ent = [struct.unpack_from("<QIBB", s, 64 + 16 * i) for i in range(nch * G)]
+    return [P + e[0] for e in ent if e[2] in (1, SPARSE) and s[P + e[0]:P + e[0] + 12] == bytes(12)]
+
+
+FLAT = [("u8", 0.1), ("u8", 0.3), ("u8", 0.6), ("u8", 0.9), ("fp16", 0.3), ("fp16", 0.6),
+        ("fp32", 0.3), ("fp32", 0.6), ("fp32", 0.9)]
+
+
+@pytest.mark.parametrize("kind,live", FLAT)
+def test_oracle_codes_uniform_live_bytes(kind, live):
+    x = pruned(kind, 3 * 16384 + 55, live, 800)
+    s = O.compress(x, CODE[kind], 262144)
+    at = flat_groups(s)
+    assert at and all(s[a + 12:a + 268] == bytes(range(256)) for a in at)
+    assert np.array_equal(O.decompress(s), x)
+    for k in (12, 77, 267):                  # any other symbols under zero counts: refused
+        bad = bytearray(s)
+        bad[at[0] + k] ^= 1
+        with pytest.raises(O.OracleError):
+            O.decompress(bytes(bad))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind,live", FLAT)
+def test_uniform_live_bytes(kind, live):
+    from paper_2411_05239_gb300 import zipnn as Z
+    dt = CODE[kind]
+    x = pruned(kind, 3 * 16384 + 55, live, 800)
+    t = torch.from_numpy(x).cuda().view(Z.CODE_TO_TORCH[dt])
+    want = O.compress(x, dt, 262144, Z.default_lanes(dt, 262144))
+    c = Z.compress(t)
+    assert c.to_bytes() == want
+    decode_every_way(c, t)
+    for k in (12, 77, 267):
+        bad = torch.frombuffer(bytearray(want), dtype=torch.uint8).cuda()
+        bad[flat_groups(want)[0] + k] ^= 1
+        out = torch.empty_like(t)
+        Z.decompress(Z.wrap(bad, bad.numel()), out)
+        with pytest.raises(Z.ZipnnError) as e:
+            Z.sync_status()
+        assert e.value.status == -3

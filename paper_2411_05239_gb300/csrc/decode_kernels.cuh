@@ -141,7 +141,8 @@ struct ChunkInfo {
   // staged payloads, as shared-window addresses (of byte 0 of what may be
   // staged in part: the vector bitmap, the start-bit table, the bitstream)
   uint32_t at_bm[4], at_starts[4], at_words[4];
-  uint32_t end[4];          // where readers of the bitstream are clamped
+  uint32_t end[4];          // where readers of the bitstream are clamped,
+  uint32_t first[4];        // and the first bit of it in the stage
   uint32_t lut[4];          // shared-window address of the group's table
   uint32_t coded;           // bit g: group g is coded (HUFF or SPARSE)
   uint32_t pairs;           // bit g: its table holds pairs
@@ -603,7 +604,7 @@ __device__ __forceinline__ void decode_weights(const Smem& S, uint32_t lut, uint
       const uint32_t t = t0 + j * nthr < t_b ? t0 + j * nthr : t0;
       v[j] = t;
       uint32_t start = t ? lds32v(starts + 4u * (t - 1)) : 0u;
-      if (start > nbits) {
+      if (start > nbits || start < CI.first[0]) {
         bad = kBad;
         start = nbits;
       }
@@ -799,7 +800,7 @@ __device__ __forceinline__ void decode_general(const Smem& S, uint32_t* err, uin
     for (int g = 0; g < G; g++) {
       if (!((coded >> g) & 1u)) continue;
       uint32_t start = t ? start_of(g, t) : 0u;
-      if (start > CI.nwords[g] * 32u) {
+      if (start > CI.nwords[g] * 32u || (WH == kStaged && start < CI.first[g])) {
         bad = kBad;
         start = CI.nwords[g] * 32u;
       }
@@ -1027,6 +1028,7 @@ __device__ __forceinline__ void setup_item(Smem& S, uint32_t parts, uint32_t lut
       CI.at_starts[g] = at + h + bmb;
       CI.at_words[g] = at + hdr;
       CI.end[g] = at + hdr + 4u * (nw + 4u);
+      CI.first[g] = 0;
     }
   }
   uint32_t slots = 0, threads = 0;
@@ -1092,6 +1094,7 @@ __device__ __noinline__ uint32_t stage_slice(Smem& S, uint32_t t_a, uint64_t* ba
                           CI.offs[g];
         CI.at_words[g] = piece(g, CI.bs[g] + 4u * w0, CI.bs[g] + 4u * w1) + CI.bs[g];
         CI.end[g] = CI.at_words[g] + 4u * (w1 + 3u);
+        CI.first[g] = 32u * w0;
       }
       total = to - CI.stage;
       if (pass == 0) {

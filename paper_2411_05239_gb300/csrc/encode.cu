@@ -129,11 +129,14 @@ __device__ __forceinline__ void split_vec(int dtype, uint4 a, uint32_t out[4][4]
 
 // ---------------------------------------------------------------------------
 // The encoder's kernels follow one another on a stream as programmatic
-// dependents: each lets the next one's CTAs start once its own are all
-// running (next_may_start), and each waits for the whole grid before it, memory
-// included, before it reads what that wrote.  A launch then costs its successor
-// little: a 48 KiB tensor takes 27.7 us like this and 31.2 with plain
-// launches, an 8 MiB one 37.4 and 45.7.
+// dependents: k_hist and k_build let the next one's CTAs start once their own are
+// all running (next_may_start), and each kernel waits for the whole grid before it,
+// memory included, before it reads what that wrote.  A launch then costs its
+// successor little: a 48 KiB tensor takes 25.6 us like this and 31.2 with plain
+// launches, an 8 MiB one 37.9 and 45.7.  k_scan does not let k_pack start: its CTAs
+// would take their places while the kernels before it still hold some SMs, two on
+// one SM and none on another, which costs launches of fewer chunks than two per SM
+// a quarter (16 MiB of BF16 49 us, now 37.4; 38 MiB of U8 173, now 135).
 
 __device__ __forceinline__ void next_may_start() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -870,7 +873,6 @@ constexpr int kScanThreads = 1024;
 __global__ void __launch_bounds__(kScanThreads)
 k_scan(JobRef jr, GcMeta* meta, uint64_t* offs, uint64_t* totals, uint32_t* err) {
   __shared__ uint64_t warp_sums[kScanThreads / 32];
-  next_may_start();
   wait_before(meta);
   const int j = blockIdx.x;
   const Job& J = job_at(jr, j);

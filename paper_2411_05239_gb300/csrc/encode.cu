@@ -1692,11 +1692,11 @@ __device__ __forceinline__ void write_map_entries(const Job& J, uint64_t c, cons
 // Packing of chunk c whose mode records (S.meta), payload offsets (S.off) and
 // codes of its coded groups (S.codes) are in shared memory and whose map
 // entries have been written; tabp[g] points to group g's table bytes.
-template <int DT, bool S2 = false>
+template <int DT, bool S2 = false, bool BIG = false>
 __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t* slots,
                                 const uint8_t* const* tabp);
 
-template <int DT, bool S2 = false>
+template <int DT, bool S2 = false, bool BIG = false>
 __device__ void pack_chunk(const Job& J, uint64_t c, PackSmem& S, uint32_t* slots,
                            const uint32_t* codes, const uint8_t* tabs, const GcMeta* meta,
                            const uint64_t* offs) {
@@ -1727,7 +1727,7 @@ __device__ void pack_chunk(const Job& J, uint64_t c, PackSmem& S, uint32_t* slot
   const uint8_t* tabp[4] = {nullptr, nullptr, nullptr, nullptr};  // null: written
 #pragma unroll
   for (int g = 1; g < G; g++) tabp[g] = tabs + (gc0 + g) * kTabBytes;
-  pack_chunk_core<DT, S2>(J, c, S, slots, tabp);
+  pack_chunk_core<DT, S2, BIG>(J, c, S, slots, tabp);
 }
 
 // Pass B of a chunk whose group 0 is its only coded group and whose units
@@ -1769,9 +1769,11 @@ __device__ __forceinline__ void pass_b_whole(const PackSmem& S, const uint32_t* 
 }
 
 // The same for units of any size that fits their slots of cap words at sl0 (a
-// word may span several units), offsets in part[0..units].
+// word may span several units, but two at most when all hold 32 bits or more: big),
+// offsets in part[0..units].
 __device__ __forceinline__ void pass_b_any(const uint32_t* part, uint32_t sl0, uint32_t cap,
-                                           uint32_t units, uint32_t* words, uint32_t capw) {
+                                           uint32_t units, uint32_t* words, uint32_t capw,
+                                           bool big) {
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, nwarps = nthr >> 5;
   const uint32_t tot = part[units], used = min((tot + 31u) >> 5, capw);
   const uint32_t upw = (units + (uint32_t)nwarps - 1) / (uint32_t)nwarps;
@@ -1790,11 +1792,15 @@ __device__ __forceinline__ void pass_b_any(const uint32_t* part, uint32_t sl0, u
       const uint32_t a = lds32v(sl + 4u * i);
       const uint32_t b = 32u * (i + 1) < e - o ? lds32v(sl + 4u * (i + 1)) : 0u;
       uint32_t x = __funnelshift_l(b, a, k & 31), r = e - bit, ee = e;
-      for (uint32_t nu = cu + 1; r < 32 && nu < units; nu++) {
-        const uint32_t e2 = part[nu + 1];
-        if (e2 > ee) x |= lds32v(sl0 + 4u * nu * cap) >> r;
-        r += e2 - ee;
-        ee = e2;
+      if (big) {
+        if (r < 32 && cu + 1 < units) x |= lds32v(sl + 4u * cap) >> r;
+      } else {
+        for (uint32_t nu = cu + 1; r < 32 && nu < units; nu++) {
+          const uint32_t e2 = part[nu + 1];
+          if (e2 > ee) x |= lds32v(sl0 + 4u * nu * cap) >> r;
+          r += e2 - ee;
+          ee = e2;
+        }
       }
       words[w] = x;
     }
@@ -1802,7 +1808,7 @@ __device__ __forceinline__ void pass_b_any(const uint32_t* part, uint32_t sl0, u
   for (uint32_t w = used + tid; w < capw; w += nthr) words[w] = 0;
 }
 
-template <int DT, bool S2>
+template <int DT, bool S2, bool BIG>
 __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t* slots,
                                 const uint8_t* const* tabp) {
   constexpr int G = PTraits<DT>::G, V = PTraits<DT>::V, ES = 16 / V;
@@ -2043,17 +2049,27 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
   // pass_b_whole when there is one group, HUFF (a SPARSE one has its bitmap before
   // the starts, and empty units), 32 bits or more in every unit (so that a
   // word spans at most two) and a unit per thread or FP32 (256 MiB: 229.6 us
-  // against 232.7; a second copy of it costs the 16-bit kernels more in
-  // registers than it gains with several units a thread), else pass_b_any
-  bool whole = sg == 0 && huff == 1u && sparse == 0;
+  // against 232.7), else pass_b_any, which units of 32 bits or more let look at two
+  // units only (BIG: 16-bit launches; 256 lanes, encode of 3.0 GB: 1788 -> 1742 us.  In
+  // the kernel for several types it costs more in registers than it gains.)
+  // (Each thread looks at its own units: nothing has waited for the other threads yet.)
+  const bool single = sg == 0 && huff == 1u && sparse == 0;
+  bool fit = huff == ((sg >= 0 ? 1u << sg : 0u) | (sg1 >= 0 ? 1u << sg1 : 0u));
+  bool whole = BIG ? fit : single;
   // one unit per thread (unit tid): its exclusive bit offset from a warp scan
   // before this barrier and a scan of the warp totals after it
-  const bool one = R == 1 && units == (uint32_t)nthr;
+  const bool one = R == 1 && units == (uint32_t)nthr && (!BIG || single);
   const int lane = tid & 31, wid = tid >> 5;
   uint32_t ub = 0, uincl = 0;
+  if (BIG)
+    for (uint32_t u = tid; fit && u < units; u += nthr) {
+      const uint32_t b = S.sbits[gmod(u, T) * R + gdiv(u, T)];
+      fit = b <= slot_cap * 32u;
+      whole = whole && fit && b >= 32u;
+    }
   if (one) {
     ub = S.sbits[tid];
-    whole = whole && ub >= 32u && ub <= slot_cap * 32u;
+    if (!BIG) whole = whole && ub >= 32u && ub <= slot_cap * 32u;
     uincl = ub;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -2062,12 +2078,11 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
     }
     if (lane == 31) S.wsum[wid] = uincl;
   } else if (DT == ZIPNN_FP32) {
-    // (this thread's own units: nothing has waited for the other threads yet)
     for (uint32_t u = tid; whole && u < units; u += nthr) {
       const uint32_t b = S.sbits[gmod(u, T) * R + gdiv(u, T)];
       whole = b >= 32u && b <= slot_cap * 32u;
     }
-  } else {
+  } else if (!BIG) {
     whole = false;
   }
   whole = __syncthreads_and(whole) != 0;
@@ -2094,10 +2109,10 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
     return;
   }
 
-  bool fit = (DT == ZIPNN_FP32 && whole) || huff == ((sg >= 0 ? 1u << sg : 0u) | (sg1 >= 0 ? 1u << sg1 : 0u));
-  for (uint32_t u = tid; fit && !(DT == ZIPNN_FP32 && whole) && u < units; u += nthr)
-    fit = S.sbits[u] <= slot_cap * 32u && (sg1 < 0 || S.part[sg1 < 0 ? 0 : sg1][u] <= slot_cap1 * 32u);
-  fit = __syncthreads_and(fit) != 0;
+  if (!BIG)
+    for (uint32_t u = tid; fit && !whole && u < units; u += nthr)
+      fit = S.sbits[u] <= slot_cap * 32u && (sg1 < 0 || S.part[sg1 < 0 ? 0 : sg1][u] <= slot_cap1 * 32u);
+  fit = __syncthreads_and(fit || whole) != 0;
 
   // scan unit bits -> unit offsets; table bytes, sub-stream starts, zeroed words
 #pragma unroll
@@ -2133,7 +2148,8 @@ __device__ void pack_chunk_core(const Job& J, uint64_t c, PackSmem& S, uint32_t*
     for (int g = 0; g < G; g++)
       if (g == sg || (S2 && g == sg1))
         pass_b_any(S.part[g], g == sg ? smem_u32(slots) : slots1, g == sg ? slot_cap : slot_cap1, units,
-                   reinterpret_cast<uint32_t*>(out + P + S.off[g] + S.hsz[g]), S.capw[g]);
+                   reinterpret_cast<uint32_t*>(out + P + S.off[g] + S.hsz[g]), S.capw[g],
+                   BIG && whole);
     return;
   }
 
@@ -2274,7 +2290,8 @@ k_pack(JobRef jr, uint64_t nchunks_total, const uint32_t* codes, const uint8_t* 
   if (totals[j] > J.out_capacity) return;
   const uint64_t c = chunk - J.chunk_begin;
   if (DTS >= 0) {
-    pack_chunk<(DTS < 0 ? 0 : DTS), S2>(J, c, S, slots, codes, tabs, meta, offs);
+    pack_chunk<(DTS < 0 ? 0 : DTS), S2, !S2 && (DTS == ZIPNN_BF16 || DTS == ZIPNN_FP16)>(
+        J, c, S, slots, codes, tabs, meta, offs);
     return;
   }
   switch (J.dtype) {

@@ -53,16 +53,15 @@ DecodeConfig decode_config(const DecodeShape& sh, int threads, uint64_t items_pe
   // (12 bits a symbol), the bitmap, and what its pieces are rounded to.  FP32 weights
   // slice chunks of one HUFF group only, which need no other table (kReadsDirect).
   const uint64_t vecs = (sh.max_chunk / 16 + sh.min_lanes - 1) / sh.min_lanes;
-  const uint64_t slice =
-      fp32 && c.kind == kWeights
-          ? vecs * 6 + 192
-          : tabs + vecs * 24 + (sh.max_chunk / 128 + 192) * (uint64_t)sh.max_groups;
+  const uint64_t fixed =
+      fp32 && c.kind == kWeights ? 192 : tabs + (sh.max_chunk / 128 + 192) * (uint64_t)sh.max_groups;
+  const uint64_t slice = fixed + vecs * (fp32 && c.kind == kWeights ? 6 : 24);
   const uint32_t two = 2u * (256u / (uint32_t)threads);
   const uint32_t least = items_per_sm >= two ? two : (items_per_sm ? (uint32_t)items_per_sm : 1u);
   // (the register budgets of the kernels, see kernel_of)
   uint32_t ctas = threads == 256 && (!fp32 || c.kind == kWeights) ? 3u : two;
   while (ctas > least && cap(ctas) < want) ctas--;
-  while (ctas > 1u && (cap(ctas) < slice || cap(ctas) + c.ring < tabs)) ctas--;
+  while (ctas > 1u && (cap(ctas) < fixed || cap(ctas) + c.ring < tabs)) ctas--;
   const uint64_t room = cap(ctas);
   const bool over = want > room + (sh.general ? 0 : room / 8);
   if (sh.family == ZIPNN_U8 || (over && (!sh.stage_need || sh.general)) || room < slice) {

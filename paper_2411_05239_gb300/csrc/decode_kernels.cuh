@@ -554,7 +554,7 @@ __device__ __forceinline__ void decode_weights(const Smem& S, uint32_t lut, uint
   Source<kStaged> src;
   src.base = CI.at_words[0];
   src.end = CI.end[0];
-  const uint32_t nbits = CI.nwords[0] * 32u;
+  const uint32_t nbits = CI.nwords[0] * 32u, first = CI.first[0];
   const bool pairs = CI.pairs & 1u;
   uint32_t rawm = 0;
   uint32_t cw[G];
@@ -604,7 +604,7 @@ __device__ __forceinline__ void decode_weights(const Smem& S, uint32_t lut, uint
       const uint32_t t = t0 + j * nthr < t_b ? t0 + j * nthr : t0;
       v[j] = t;
       uint32_t start = t ? lds32v(starts + 4u * (t - 1)) : 0u;
-      if (start > nbits || start < CI.first[0]) {
+      if (start - first > nbits - first) {
         bad = kBad;
         start = nbits;
       }
@@ -943,7 +943,7 @@ __device__ __forceinline__ void setup_item(Smem& S, uint32_t parts, uint32_t lut
   }
   const bool fits = total + 32u <= room;
   // (DIRECT: what does not take the weight loop is read from global memory)
-  const bool direct = DIRECT && !__shfl_sync(0xffffffffu, coded == 1u && mode == kHuff, 0);
+  const bool direct = DIRECT && !(coded == 1u && (S.entry[0].w & 0xFFu) == kHuff);
   const uint32_t at = stage0 + extra + (uint32_t)before;
   if (lane < (uint32_t)G) {
     const uint32_t k = (uint32_t)__popc(coded & ((1u << lane) - 1u));
@@ -982,12 +982,7 @@ __device__ __forceinline__ void setup_item(Smem& S, uint32_t parts, uint32_t lut
     if (i2 < 68u) t.words[i2] = b2;
     const uint32_t cword = __shfl_sync(0xffffffffu, b0, ((lane - 1u) >> 2) & 3u);
     const bool is_len = lane >= 1u && lane <= (uint32_t)kMaxLen;
-    // 256 codes of 8 bits, whose count is stored as 0: twelve zeros, symbols 0..255
-    auto flat = [](uint32_t i) { return i < 3u ? 0u : 0x03020100u + 0x04040404u * (i - 3u); };
-    const bool all8 = __all_sync(0xffffffffu, b0 == flat(lane) && b1 == flat(i1) &&
-                                                  (i2 > 66u || b2 == flat(i2)));
-    const uint32_t cl = all8 && lane == 8u ? 256u
-                        : is_len ? (cword >> (8u * ((lane - 1u) & 3u))) & 0xFFu : 0u;
+    const uint32_t cl = is_len ? (cword >> (8u * ((lane - 1u) & 3u))) & 0xFFu : 0u;
     const uint32_t A = is_len ? cl << (kMaxLen - lane) : 0u;
     uint32_t lim = A, idx = cl;
 #pragma unroll
@@ -1003,7 +998,14 @@ __device__ __forceinline__ void setup_item(Smem& S, uint32_t parts, uint32_t lut
       t.rank[lane] = (idx - cl) - ((lim - A) >> (kMaxLen - lane));
     }
     const uint32_t kraft = __shfl_sync(0xffffffffu, lim, kMaxLen);
-    const uint32_t nz = __shfl_sync(0xffffffffu, idx, kMaxLen);
+    uint32_t nz = __shfl_sync(0xffffffffu, idx, kMaxLen);
+    if (nz == 0) {  // 256 codes of 8 bits, whose count is stored as 0? (then the symbols are 0..255)
+      auto flat = [](uint32_t i) { return i < 3u ? 0u : 0x03020100u + 0x04040404u * (i - 3u); };
+      if (__all_sync(0xffffffffu, b0 == flat(lane) && b1 == flat(i1) && (i2 > 66u || b2 == flat(i2)))) {
+        nz = 256;
+        if (is_len && lane >= 8u) t.lim[lane] = (uint32_t)kLutSize;
+      }
+    }
     // windows that hold two whole codes: for a first code of length l, the
     // codes of at most 12 - l bits
     const uint32_t rest = __shfl_sync(0xffffffffu, lim, (kMaxLen - lane) & 31u);
@@ -1225,9 +1227,10 @@ __device__ __forceinline__ void decode_range(const Smem& S, uint32_t lut0, uint3
 // CTAs per SM that the registers are budgeted for: three (80 registers), or two
 // (128) where the stage leaves no room for three, where the general loop over
 // four groups would spill (what spills misses the 28 KiB of L1 that the shared
-// memory leaves), and in the 128-thread kernels of small launches.
+// memory leaves), and in the 128-thread kernels of small launches.  (The tables of
+// FP32 weights leave room for three of 128 threads at most.)
 template <int DT, int KIND, int NT, int REGS>
-__global__ void __launch_bounds__(NT, REGS * 256 / NT)
+__global__ void __launch_bounds__(NT, DT == ZIPNN_FP32 && KIND == kWeights ? 3 : REGS * 256 / NT)
 k_decode(JobRef jr, uint64_t nchunks_total, uint32_t* __restrict__ err,
          unsigned long long* __restrict__ ticket, uint32_t debug_flags, uint32_t ntab,
          uint32_t stage_cap, uint32_t ring_bytes, uint32_t pf_bytes, uint32_t parts) {

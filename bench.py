@@ -287,20 +287,20 @@ def run_gb300(args):
     ts = W.checkpoint_bf16(specs, seed=2, device=dev)
     orig = sum(t.numel() * 2 for t in ts)
 
-    # autotuned container (chunk size, lanes) and decoder (table width, CTAs/SM)
+    # autotuned container (chunk size, lanes) and decoder (CTA size, CTAs/SM)
     # settings, measured on a sample of the checkpoint (embedding rows + 2 layers)
     tuned = None
     lanes = args.lanes
     if args.autotune:
         # the autotuner sweeps chunk sizes 64 KiB - 1 MiB (container), lanes,
-        # table width, CTA size and CTAs per SM (decoder) on a sample and caches
+        # CTA size and CTAs per SM (decoder) on a sample and caches
         # the winner for this workload (GPU, dtype, size class); the library's
         # Python API then takes the cached setting itself: the compressor below
         # is given no chunk size and the decode plan no tuning
         from paper_2411_05239_gb300 import autotune as AT
         sample = [ts[0][: 64 * 1024 * 1024]] + ts[1:1 + 2 * 9]
         tuned = AT.tuned(sample, nbytes=orig, force=not args.autotune_cache, reps=3,
-                         chunks=AT.CHUNKS, lut_bits=(11, 12), ctas=(0, 2, 3))
+                         chunks=AT.CHUNKS, ctas=(0, 2, 3))
         if args.autotune_log and "table" in tuned:
             with open(args.autotune_log, "w") as f:
                 json.dump(tuned["table"], f)

@@ -394,8 +394,8 @@ __device__ __forceinline__ uint32_t quad_singles(Bits& r, const Source<WH>& s, u
   return __byte_perm(a, b, 0x5410);
 }
 
-// merge16 / merge32 for exponent bytes stored rotated right by one bit
-// (e' = e >> 1 | e << 7 per byte): each output byte is a bit select.
+// The inverses of split16 / split32 for exponent bytes stored rotated right by one
+// bit (e' = e >> 1 | e << 7 per byte): each output byte is a bit select.
 __device__ __forceinline__ void merge16r(uint32_t er, uint32_t r, uint32_t& w0, uint32_t& w1) {
   const uint32_t hi = (r & 0x80808080u) | (er & 0x7F7F7F7Fu);
   const uint32_t lo = (er & 0x80808080u) | (r & 0x7F7F7F7Fu);
@@ -1407,7 +1407,7 @@ const void* kernel_of(int threads, bool three) {
   if constexpr (DT != ZIPNN_FP32 || KIND == kWeights)
     if (three || DT != ZIPNN_BF16 || KIND == kRings)
       return reinterpret_cast<const void*>(k_decode<DT, KIND, 256, 3>);
-  if constexpr (DT == ZIPNN_BF16 || (DT == ZIPNN_FP32 && KIND != kWeights))
+  if constexpr ((DT == ZIPNN_BF16 && KIND != kRings) || (DT == ZIPNN_FP32 && KIND != kWeights))
     return reinterpret_cast<const void*>(k_decode<DT, KIND, 256, 2>);
   return nullptr;
 }

@@ -111,14 +111,6 @@ __device__ __forceinline__ void split16(uint32_t w0, uint32_t w1, uint32_t& e, u
   r = (hi & 0x80808080u) | (lo & 0x7F7F7F7Fu);
 }
 
-// Inverse of split16 for 4 elements: bytes e (g0) and r (g1) -> two u32 words.
-__device__ __forceinline__ void merge16(uint32_t e, uint32_t r, uint32_t& w0, uint32_t& w1) {
-  uint32_t hi = (r & 0x80808080u) | ((e >> 1) & 0x7F7F7F7Fu);
-  uint32_t lo = ((e << 7) & 0x80808080u) | (r & 0x7F7F7F7Fu);
-  w0 = __byte_perm(lo, hi, 0x5140);  // L0 H0 L1 H1
-  w1 = __byte_perm(lo, hi, 0x7362);  // L2 H2 L3 H3
-}
-
 // FP32 element x: g0 = x >> 23 & 0xFF, g1 = (x >> 24 & 0x80) | (x >> 16 & 0x7F),
 // g2 = x >> 8 & 0xFF, g3 = x & 0xFF.  Four elements -> one u32 per group.
 __device__ __forceinline__ void split32(const uint32_t x[4], uint32_t g[4]) {
@@ -131,21 +123,6 @@ __device__ __forceinline__ void split32(const uint32_t x[4], uint32_t g[4]) {
   g[1] = (b3 & 0x80808080u) | (b2 & 0x7F7F7F7Fu);
   g[2] = b1;
   g[3] = b0;
-}
-
-__device__ __forceinline__ void merge32(const uint32_t g[4], uint32_t x[4]) {
-  uint32_t b3 = (g[1] & 0x80808080u) | ((g[0] >> 1) & 0x7F7F7F7Fu);
-  uint32_t b2 = ((g[0] << 7) & 0x80808080u) | (g[1] & 0x7F7F7F7Fu);
-  uint32_t b1 = g[2], b0 = g[3];
-  // element k bytes (b0_k, b1_k, b2_k, b3_k) little-endian
-  uint32_t lo01 = __byte_perm(b0, b1, 0x5140);  // b0_0 b1_0 b0_1 b1_1
-  uint32_t hi01 = __byte_perm(b2, b3, 0x5140);  // b2_0 b3_0 b2_1 b3_1
-  uint32_t lo23 = __byte_perm(b0, b1, 0x7362);
-  uint32_t hi23 = __byte_perm(b2, b3, 0x7362);
-  x[0] = __byte_perm(lo01, hi01, 0x5410);
-  x[1] = __byte_perm(lo01, hi01, 0x7632);
-  x[2] = __byte_perm(lo23, hi23, 0x5410);
-  x[3] = __byte_perm(lo23, hi23, 0x7632);
 }
 
 }  // namespace zipnn

@@ -13,7 +13,8 @@
 //      TMA bulk copy each (cp.async.bulk, completion on an mbarrier; payloads
 //      are 16-B aligned and padded by the format) and derives the canonical
 //      limits of each coded group with warp scans; the ticket and the map
-//      entries were requested while the item before this one was set up,
+//      entries were requested while the item before this one was set up (payloads
+//      that the stage cannot hold: see Where and stage_slice),
 //   2. all warps build, per coded group, a 4096-entry table indexed by the
 //      next 12 bits (12 = the longest code): the first code of the window, and
 //      both its first codes when they fit in it and the group's code makes
